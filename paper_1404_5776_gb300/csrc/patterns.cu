@@ -45,6 +45,15 @@ void* Arena::get(size_t bytes) {
   return p;
 }
 
+void Arena::put(void* p) {
+  for (size_t k = 0; k < blocks.size(); ++k)
+    if (blocks[k] == p) {
+      alloc->put(p, stream);
+      blocks.erase(blocks.begin() + k);
+      return;
+    }
+}
+
 void Arena::release_all() {
   for (void* p : blocks) alloc->put(p, stream);
   blocks.clear();

@@ -45,6 +45,7 @@ struct TripleKey {
 };
 
 struct TripleInfo {
+  const Pattern *pa = nullptr, *pb = nullptr;  // the operands' patterns
   Triples t;
   TileList tiles;  // row tiles for the tensor-core kernel (built for the sandwich's FP32 13-function products)
   int64_t true_macs = 0;
@@ -158,6 +159,12 @@ struct rt_ctx {
   std::vector<std::unique_ptr<rt::Sys>> sys;
   rt::FieldParams field;
   rt::DevState* dstate = nullptr;
+  // split operands of the FP64 13-function products (op(A), op(B)): one pair for
+  // the context, whose products run one after another on its stream; sized for
+  // the largest pattern and grown outside a capture
+  rt::X64Operand xa, xb;
+  size_t xa_bytes = 0, xb_bytes = 0;
+  int x_atoms = 0;
   void* zero32 = nullptr;  // one zero FP32 complex block (padded layout)
   int* d_err = nullptr;    // device error word of bounded waits
   long long wait_ns = 2000000000ll;  // budget of one bounded device wait
@@ -266,6 +273,8 @@ static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* 
   auto ti = std::make_unique<TripleInfo>();
   build_triples(ti->t, *A, ad, *B, bd, *C, up, c->arena, c->ws);
   ti->true_macs = triple_true_macs(ti->t, *A, ad, *C, s.d_bsize, c->arena, c->ws);
+  ti->pa = A;
+  ti->pb = B;
   ti->nnzb_a = A->nnzb;
   ti->nnzb_b = B->nnzb;
   auto elems = [&](const Pattern* P) {
@@ -362,10 +371,67 @@ static GemmArgs prepared(rt_ctx* c, Sys& s, TripleInfo& ti, bool fp32, bool cplx
   return g;
 }
 
+// Room for the split operands of a product over patterns of at most nnzb blocks.
+static void reserve_split(rt_ctx* c, const Sys& s, int64_t nnzb_a, int64_t nnzb_b, bool cplx) {
+  const size_t na = (size_t)nnzb_a * x64_block_bytes(cplx), nb = (size_t)nnzb_b * x64_block_bytes(cplx);
+  if (na <= c->xa_bytes && nb <= c->xb_bytes && s.n_atoms <= c->x_atoms) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  RT_CUDA_CHECK(cudaStreamIsCapturing(c->ws, &cs));
+  RT_REQUIRE(cs == cudaStreamCaptureStatusNone, RT_EINTERNAL, "split operands must be sized before a capture");
+  auto grow = [&](auto*& p, size_t& have, size_t want) {
+    if (want <= have) return;
+    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+    using T = std::remove_reference_t<decltype(*p)>;
+    if (p) c->arena.put(p);
+    p = nullptr;
+    have = 0;
+    p = static_cast<T*>(c->arena.get(want));
+    have = want;
+  };
+  size_t la = c->xa_bytes / x64_block_bytes(false), lb = c->xb_bytes / x64_block_bytes(false);
+  grow(c->xa.lead, la, na / x64_block_bytes(false));
+  grow(c->xb.lead, lb, nb / x64_block_bytes(false));
+  grow(c->xa.dig, c->xa_bytes, na);
+  grow(c->xb.dig, c->xb_bytes, nb);
+  size_t ea = (size_t)c->x_atoms * 64, eb = ea;
+  const size_t ne = (size_t)std::max(s.n_atoms, c->x_atoms) * 64;
+  grow(c->xa.exps, ea, ne);
+  grow(c->xb.exps, eb, ne);
+  c->x_atoms = std::max(s.n_atoms, c->x_atoms);
+  c->graph_dirty = true;  // a captured step holds the old addresses
+}
+
+// Gives the split operands back: in a mixed-precision EM, ETRS or M4 context only
+// the set-up has FP64 products, and at 10 A and 4096 atoms the two take 12.7 GB.
+static void release_split(rt_ctx* c) {
+  if (!c->xa.dig && !c->xb.dig) return;
+  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+  for (X64Operand* x : {&c->xa, &c->xb}) {
+    for (void* p : {(void*)x->dig, (void*)x->lead, (void*)x->exps})
+      if (p) c->arena.put(p);
+    *x = X64Operand();
+  }
+  c->xa_bytes = c->xb_bytes = 0;
+  c->x_atoms = 0;
+}
+
+// keep_a: A is the operand of the product just before, unchanged since, so that its split stands
 static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cplx, bool ad, bool bd, Epilogue epi,
-                 GemmArgs g, const Pattern* C) {
+                 GemmArgs g, const Pattern* C, bool keep_a = false) {
   g = prepared(c, s, ti, fp32, cplx, epi, g, C);
   int B = s.B;
+  if (B == 13 && !fp32) {
+    if (!c->counting) reserve_split(c, s, ti.nnzb_a, ti.nnzb_b, cplx);
+    run(
+        c, cls, gemm_flops(ti, cplx), gemm_bytes(s, ti, cplx, fp32),
+        [&] {
+          if (!keep_a) launch_split13(g.A, cplx, ad, false, *ti.pa, c->xa, c->ws);
+          launch_split13(g.B, cplx, !bd, true, *ti.pb, c->xb, c->ws);
+          launch_gemm13_x64(cplx, ad, bd, epi, g, c->xa, c->xb, c->ws);
+        },
+        keep_a ? 2 : 3);
+    return;
+  }
   RT_REQUIRE(!g.a_planar || (fp32 && cplx && B == 13 && !ti.tiles.built), RT_EINTERNAL,
              "column-planar operands belong to the packed CUDA-core products");
   RT_REQUIRE(!g.kf32 || (fp32 && cplx && epi == EPI_DELTA_SANDWICH && !ti.tiles.built), RT_EINTERNAL,
@@ -670,6 +736,12 @@ static void setup_system(rt_ctx* c, Sys& s, const rt_system& in) {
       s.planar = p.packed_fma != 0 && !p.tensor_cores;
     }
   }
+  if (s.B == 13 && (p.precision == RT_FP64 || p.prop == RT_PROP_CN)) {
+    // the captured step holds FP64 products: their split operands are sized here
+    int64_t most = 0;
+    for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
+    reserve_split(c, s, most, most, true);
+  }
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
 
@@ -732,7 +804,7 @@ static rt_status hotelling_sinv(rt_ctx* c, Sys& s) {
     // T0 = cut(S^-1 H0) and T_D = cut(S^-1 D_dir): T(t) = T0 - E(t) T_D exactly
     TripleInfo& tT = triples_for(c, s, P, false, s.pH, false, s.pT, false);
     gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.H0, s.T0), s.pT);
-    gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.D[c->field.dir], s.TD), s.pT);
+    gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.D[c->field.dir], s.TD), s.pT, true);
   }
   if (c->p.field_poly) build_field_poly(c, s);
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
@@ -783,7 +855,7 @@ static void taylor_series(rt_ctx* c, Sys& s, const double* T, double dt, int ter
       g.U = Uout;
       g.coef = cn;
       g.coef_imag = ci;
-      gemm(c, s, PC_TAYLOR, n == 2 ? t2 : tn, false, false, false, false, EPI_STORE_ACC, g, s.pU);
+      gemm(c, s, PC_TAYLOR, n == 2 ? t2 : tn, false, false, false, false, EPI_STORE_ACC, g, s.pU, n > 2);
       prev = bufs[n % 2];
     }
   } else {
@@ -932,7 +1004,7 @@ static void build_m4(rt_ctx* c, Sys& s, bool fp32) {
   for (int n = 2; n < p.taylor_terms; ++n) {
     inv_fact /= n;
     double2* out = bufs[n % 2];
-    gemm(c, s, PC_TAYLOR, tUU, false, true, false, false, EPI_STORE, args(s.Zc, prev, out), s.pU);
+    gemm(c, s, PC_TAYLOR, tUU, false, true, false, false, EPI_STORE, args(s.Zc, prev, out), s.pU, n > 2);
     run(c, PC_MISC, 0, 0, [&] { launch_zaxpy(s.U, s.U, out, inv_fact, nu, c->ws); });
     prev = out;
   }
@@ -953,7 +1025,7 @@ static void build_field_poly(rt_ctx* c, Sys& s) {
   const size_t nT = nvals(s, PT), nU = nvals(s, PU);
   TripleInfo& tT = triples_for(c, s, s.pSinv, false, s.pH, false, PT, false);
   gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.H0, s.T0), PT);
-  gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.D[c->field.dir], s.TDn), PT);
+  gemm(c, s, PC_MISC, tT, false, false, false, false, EPI_STORE, args(s.Sinv, s.D[c->field.dir], s.TDn), PT, true);
   launch_scale(s.TDn, -1.0, (int64_t)nT, c->ws);
   launch_identity(reinterpret_cast<double*>(s.V[0]), true, PU->nnzb, PU->rowidx, PU->col, s.B, 1.0, c->ws);
   for (int m = 1; m <= deg; ++m) RT_CUDA_CHECK(cudaMemsetAsync(s.V[m], 0, sizeof(double2) * nU, c->ws));
@@ -1208,7 +1280,7 @@ static void prepare_reference(rt_ctx* c, Sys& s) {
         gemm(c, s, PC_MISC, tM, false, true, false, false, EPI_STORE, args(s.V[m], s.Kref, Am[m]), s.pM);
       for (int m = 0; m <= deg; ++m)
         for (int m2 = 0; m2 <= deg; ++m2) {
-          gemm(c, s, PC_MISC, tK, false, true, false, true, EPI_SANDWICH, args(Am[m], s.V[m2], s.Rm), s.pK);
+          gemm(c, s, PC_MISC, tK, false, true, false, true, EPI_SANDWICH, args(Am[m], s.V[m2], s.Rm), s.pK, m2 > 0);
           launch_zaxpy(s.Bp[m + m2], s.Bp[m + m2], s.Rm, 1.0, (int64_t)nv, c->ws);
         }
       launch_zaxpy(s.Bp[0], s.Bp[0], s.Kref, -1.0, (int64_t)nv, c->ws);
@@ -1670,7 +1742,7 @@ static void ground_state(rt_ctx* c, Sys& s, int order, double mu, double kT, dou
   launch_scale(Kr, coef[0], (int64_t)nv, c->ws);
   double *Ym = Y0, *Yc = Y0, *Yn = Y1;
   for (int n = 1; n <= order; ++n) {
-    gemm(c, s, PC_MISC, tTK, false, false, false, false, EPI_STORE, args(s.T, Yc, TY), PK);
+    gemm(c, s, PC_MISC, tTK, false, false, false, false, EPI_STORE, args(s.T, Yc, TY), PK, n > 1);
     launch_cheb_step(TY, Yc, Ym, Yn, Kr, a, w, coef[n], n == 1 ? 1 : 0, (int64_t)nv, c->ws);
     // rotate: (Ym, Yc) <- (Yc, Yn); Yn <- a free buffer
     double* freeb = (n == 1) ? Y2 : Ym;
@@ -2134,6 +2206,7 @@ rt_status rt_step(rt_ctx* c, int32_t n) {
     if (n == 0) return RT_OK;
     if (incremental(c))
       for (auto& sp : c->sys) prepare_reference(c, *sp);
+    if (c->p.precision == RT_FP32 && c->p.prop != RT_PROP_CN) release_split(c);
     build_groups(c);
     if (c->inject & RT_FAULT_WAIT_TIMEOUT_0) {
       // one step, launched directly, with a zero wait budget; the error word

@@ -63,6 +63,7 @@ struct Arena {
   std::vector<void*> blocks;
   size_t total = 0;
   void* get(size_t bytes);
+  void put(void* p);  // gives one buffer back (the stream is done with it)
   template <typename T>
   T* get_n(size_t n) {
     return static_cast<T*>(get(n * sizeof(T) + 16));
@@ -213,6 +214,23 @@ inline int sb32(int B) { return B * rs32(B); }
 // epilogues EPI_STORE (and W = K + M) and EPI_DELTA_SANDWICH; false if `epi`
 // is not one of them.
 bool launch_gemm13_tc(Epilogue epi, const GemmArgs& g, cudaStream_t st);
+
+// FP64 products of 13-function atoms on the tensor cores (spgemm13_x64.cu): an
+// operand split into 64-bit fixed-point digits, one power-of-two scale per row
+// of op(A) / column of op(B), in the order in which a warp's registers take it.
+struct X64Operand {
+  unsigned char* dig = nullptr;  // [nnzb][1 real, 2 complex][4096]
+  unsigned char* lead = nullptr; // [nnzb][1 real, 2 complex] leading digits that are zero in the whole block
+  int32_t* exps = nullptr;       // [n_atoms][16] biased exponent of each scale
+};
+size_t x64_block_bytes(bool cplx);
+// The scaled index is the row of the stored blocks, or (by_col) their column:
+// op(A) takes rows as stored and columns daggered, op(B) the other way round.
+// right: the operand order of op(B).
+void launch_split13(const void* vals, bool cplx, bool by_col, bool right, const Pattern& P, const X64Operand& out,
+                    cudaStream_t st);
+void launch_gemm13_x64(bool cplx, bool a_dag, bool b_dag, Epilogue epi, const GemmArgs& g, const X64Operand& A,
+                       const X64Operand& B, cudaStream_t st);
 
 // Launches; `cplx` selects complex values, `b_dag` conj-transposes B's blocks,
 // `a_dag` A's blocks.  Element type by precision: FP64 double/double2, FP32 float/float2.

@@ -6,6 +6,8 @@
 // triples: C_ij = sum_k op(A)_ik op(B)_kj for (i,j) in P_C, k ascending.  The
 // triple lists are built once (atoms are stationary).
 //
+// FP64 products of 13-function atoms run on the tensor cores (spgemm13_x64.cu).
+//
 // Thread mapping: a group of LPB lanes owns one output block; each lane owns
 // EPL of its B*B elements and keeps them in registers.  Per triple the group
 // stages op(A)_ik and op(B)_kj (conjugate transposes applied on the way into
@@ -367,8 +369,7 @@ void launch_gemm(int B, bool fp32, bool cplx, bool a_dag, bool b_dag, Epilogue e
                         : dispatch_prec<1, double>(cplx, a_dag, b_dag, epi, g, st);
     case 4: return fp32 ? dispatch_prec<4, float>(cplx, a_dag, b_dag, epi, g, st)
                         : dispatch_prec<4, double>(cplx, a_dag, b_dag, epi, g, st);
-    case 13: return fp32 ? dispatch_prec<13, float>(cplx, a_dag, b_dag, epi, g, st)
-                         : dispatch_prec<13, double>(cplx, a_dag, b_dag, epi, g, st);
+    case 13: throw Error{RT_EINTERNAL, "FP64 13-function products take split operands (launch_gemm13_x64)"};
     default: throw Error{RT_EINVAL, "block size must pad to 1, 4 or 13"};
   }
 }

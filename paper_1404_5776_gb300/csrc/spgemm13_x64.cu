@@ -1,0 +1,532 @@
+// FP64 block products of 13-function atoms on the tensor cores.
+//
+// Same contraction as spgemm.cu (C_ij = sum_k op(A)_ik op(B)_kj over the triple
+// list of the output block).  GB300 does two FP64 fused multiply-adds per clock
+// and SM, and the CUDA-core kernel ran at 87 % of that (a real triple: 1,099
+// clocks); the tensor cores do about a thousand FP16 ones through mma.sync.  So
+// every operand is written in 64-bit fixed point and multiplied digit by digit,
+// exactly (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
+// Algorithms 59, 2012):
+//   * each row of op(A) (each column of op(B)) takes one power-of-two scale,
+//     the first power 2^e above its magnitudes over the whole block row
+//     (column); each block takes off it the whole digits that its own largest
+//     value leaves at zero (z of them): x = X 2^(e - 8 z - 62), X an integer
+//     rounded to nearest, |X| < 2^62;
+//   * X in radix 256 with digits -128..127: the bytes of X + 0x8080..80 are the
+//     digits plus 128, so the split is one 64-bit addition;
+//   * a pair of digits (p, q) has the weight p + q + z_A + z_B; the pairs of
+//     weights 0..8 are multiplied as FP16 integers (one m16n8k16 per pair and
+//     8-column half: 43 pairs with z_A + z_B = 0, 28 with two, 15 with four),
+//     each weight in its own FP32 accumulators.  One triple adds an integer of at
+//     most 13 * 8 * 2^14 to a weight, so CARRY = 8 of them stay below 2^24 and
+//     are exact; then multiples of 256 move up one weight, exactly as well;
+//   * at the end the weights meet as two 64-bit integers, and these in FP64 with
+//     one rounding.
+// Measured against quad precision on the 64- and 216-atom cells (r = 6, 8,
+// 10 A; S^-1 H and U K U^dagger): relative 2-norm error 4e-17..8e-17, where FP64
+// fused multiply-adds gave 4e-16..4e-15; the median error of single elements is
+// 7e-17..7e-16 (3e-16..2e-15 before).
+//
+// Layout: a split block is stored in the order in which an m16n8k16 operand
+// lies in a warp's registers (lane = 4 (row mod 8) + (k mod 8)/2), 16 bytes a
+// lane and load: one digit of op(A), two digits of one 8-column half of op(B).
+// Operands go from L2 straight into registers, without shared memory.  Rows and
+// k of 13..15 are padding.  One byte a digit (half the traffic, expanded in
+// registers) measured 1.03 times slower, the expansion being on the critical
+// path.
+//
+// One warp owns an 8-column half of a real output (a complex item: four warps,
+// halves x real and imaginary part, reading the same blocks through L1): 36
+// accumulators, 32 registers of A's digits and 16 of B's fit 128 registers, so
+// 16 warps a SM; a warp with both halves (168 registers, 12 warps) measured 1.3
+// times slower.  What bounds it: the tensor pipe (52-70 % busy in the Taylor
+// powers), with the wait for the next blocks' first digits beside it.
+// 216 atoms x 13, r = 8 A: a Taylor power 8.9 -> 1.14 ms with its splits, M = U K
+// 21.7 -> 3.3 ms; FP64 EM step at 512 atoms 126 -> 20.5 ms.
+#include <algorithm>
+
+#include "rt_internal.cuh"
+
+namespace rt {
+
+namespace x64 {
+
+constexpr int BS = 13;
+constexpr int NE = BS * BS;
+constexpr int BLK = 4096;      // bytes of one split real block: 8 digits x 32 lanes x 8 elements in FP16
+constexpr int WARPS = 4;
+constexpr int MINB = 4;
+constexpr int NW = 9;          // weights p + q of the digit pairs that are multiplied
+constexpr int CARRY = 8;       // real products between two carries: 13 * 8 * 2^14 * 8 + carries < 2^24
+constexpr int EXP_NAN = 2047;  // scale of a row that holds a NaN or an infinity: its products are NaN
+constexpr int MAX_LEAD = 9;    // a block with so many leading zero digits adds nothing (NW weights)
+constexpr int SPLIT_WARPS = 16;
+
+// ---------------------------------------------------------------------------
+// split: one CTA per atom; its block row (by_col: its block column, reached
+// through the transposes) is read for the scales, then again (from L2) for the
+// digits.  Bound by the integer pipe that builds the digits (58 % busy): 30 us
+// for the 31 MB of a real matrix at 216 atoms, 3 % of the product that it serves.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long fixed_biased(double x, int ex_row) {
+  const unsigned long long bias = 0x8080808080808080ull;
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7ff);
+  unsigned long long m = b & 0xfffffffffffffull;
+  if (ex) m |= 1ull << 52;
+  if (m == 0) return bias;
+  // |x| < 2^(ex_row - 1022); X = x 2^(62 - (ex_row - 1022)) = m 2^(max(ex,1) - ex_row + 9)
+  const int s = max(ex, 1) - ex_row + 9;
+  if (s >= 0) m <<= s;
+  else m = s > -64 ? (m + (1ull << (-s - 1))) >> -s : 0ull;
+  const unsigned long long v = (b >> 63) ? 0ull - m : m;
+  return v + bias;
+}
+
+__device__ __forceinline__ unsigned less_1152(unsigned h) {
+  unsigned r;
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));
+  return r;
+}
+
+template <bool CPLX>
+__global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const double* __restrict__ vals,
+                                                              const int32_t* __restrict__ rowptr,
+                                                              const int32_t* __restrict__ tmap, int by_col, int right,
+                                                              unsigned char* __restrict__ dig,
+                                                              unsigned char* __restrict__ lead,
+                                                              int32_t* __restrict__ exps) {
+  constexpr int NC = CPLX ? 2 : 1;
+  __shared__ int smax[16];
+  const int atom = blockIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int q0 = rowptr[atom], q1 = rowptr[atom + 1];
+  if (threadIdx.x < 16) smax[threadIdx.x] = 1;
+  __syncthreads();
+  constexpr int EPT = (NE + 31) / 32;
+  int mx[EPT];
+#pragma unroll
+  for (int k = 0; k < EPT; ++k) mx[k] = 1;
+  for (int q = q0 + warp; q < q1; q += SPLIT_WARPS) {
+    const double* v = vals + (int64_t)(by_col ? tmap[q] : q) * NE * NC;
+#pragma unroll
+    for (int k = 0; k < EPT; ++k) {
+      const int e = lane + 32 * k;
+      if (e < NE) {
+        int m;
+        if constexpr (CPLX) {
+          const double2 z = reinterpret_cast<const double2*>(v)[e];
+          m = max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff);
+        } else {
+          m = __double2hiint(v[e]) & 0x7fffffff;
+        }
+        mx[k] = max(mx[k], m >> 20);
+      }
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < EPT; ++k) {
+    const int e = lane + 32 * k;
+    if (e < NE) atomicMax(&smax[by_col ? e % BS : e / BS], mx[k]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 16) exps[atom * 16 + threadIdx.x] = smax[threadIdx.x];
+
+  const int g = lane >> 2, t = lane & 3;
+  for (int q = q0 + warp; q < q1; q += SPLIT_WARPS) {
+    const int qb = by_col ? tmap[q] : q;
+    const double* v = vals + (int64_t)qb * NE * NC;
+    double val[NC][8];
+#pragma unroll
+    for (int f = 0; f < 8; ++f) {
+      const int m = g + ((f >> 1) & 1) * 8;               // scaled index
+      const int k = 2 * t + (f & 1) + (f >> 2) * 8;       // summed index
+      const bool in = m < BS && k < BS && smax[m] != EXP_NAN;
+      const int e = by_col ? k * BS + m : m * BS + k;
+      if constexpr (CPLX) {
+        const double2 z = in ? reinterpret_cast<const double2*>(v)[e] : make_double2(0.0, 0.0);
+        val[0][f] = z.x;
+        val[1][f] = z.y;
+      } else {
+        val[0][f] = in ? v[e] : 0.0;
+      }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      // the block's own shift: whole digits that its largest value leaves at zero, from the
+      // exponents alone (|x| < 2^(ex - 1022) and 2^62 is the row's bound)
+      int gap = 8 * MAX_LEAD;
+#pragma unroll
+      for (int f = 0; f < 8; ++f) {
+        const int ex = (__double2hiint(val[c][f]) >> 20) & 0x7ff;
+        if (ex) gap = min(gap, smax[g + ((f >> 1) & 1) * 8] - ex);
+      }
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) gap = min(gap, __shfl_xor_sync(0xffffffffu, gap, off));
+      const int z = gap >> 3;
+      if (lane == 0) lead[(int64_t)qb * NC + c] = (unsigned char)z;
+      unsigned long long X[8];
+#pragma unroll
+      for (int f = 0; f < 8; ++f)
+        X[f] = fixed_biased(z < MAX_LEAD ? val[c][f] : 0.0, smax[g + ((f >> 1) & 1) * 8] - 8 * z);
+      uint4* out = reinterpret_cast<uint4*>(dig + ((int64_t)qb * NC + c) * BLK) + lane;
+#pragma unroll
+      for (int p2 = 0; p2 < 4; ++p2) {  // digits 2 p2 and 2 p2 + 1, most significant first
+        unsigned w[2][4];
+#pragma unroll
+        for (int d = 0; d < 2; ++d) {
+          const int p = 2 * p2 + d;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const unsigned lo = p < 4 ? (unsigned)(X[2 * r] >> 32) : (unsigned)X[2 * r];
+            const unsigned hi = p < 4 ? (unsigned)(X[2 * r + 1] >> 32) : (unsigned)X[2 * r + 1];
+            // the bytes uu of both, as the FP16 numbers 1024 + uu (0x64uu), less 1152
+            const unsigned two = __byte_perm(lo, hi, (3 - (p & 3)) | (7 - (p & 3)) << 4);  // bytes 0, 1
+            w[d][r] = less_1152(__byte_perm(two, 0x64646464u, 0x4140));
+          }
+        }
+        if (right) {
+          // op(B): the 8-column halves apart, two digits of one half together
+          out[32 * p2] = make_uint4(w[0][0], w[0][2], w[1][0], w[1][2]);
+          out[32 * (4 + p2)] = make_uint4(w[0][1], w[0][3], w[1][1], w[1][3]);
+        } else {
+          out[32 * (2 * p2)] = make_uint4(w[0][0], w[0][1], w[0][2], w[0][3]);
+          out[32 * (2 * p2 + 1)] = make_uint4(w[1][0], w[1][1], w[1][2], w[1][3]);
+        }
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
+// product
+// ---------------------------------------------------------------------------
+struct Args {
+  GemmArgs g;
+  const unsigned char* dA;
+  const unsigned char* dB;
+  const unsigned char* lA;
+  const unsigned char* lB;
+  const int32_t* eA;
+  const int32_t* eB;
+};
+
+__device__ __forceinline__ void mma16816(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
+  asm(
+      "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
+}
+// v 2^(ea - 1022) 2^(eb - 1022), a normal result by its exponent field alone; a
+// row with a NaN or an infinity gives NaN
+__device__ __forceinline__ double pow2_scaled(double v, int ea, int eb) {
+  if (ea == EXP_NAN || eb == EXP_NAN) return __longlong_as_double(0x7ff8000000000000ll);
+  const int k = ea + eb - 2044, h = __double2hiint(v), ex = ((h >> 20) & 0x7ff) + k;
+  if (v == 0.0) return 0.0;
+  return ex > 0 && ex < 2047 ? __hiloint2double(h + k * (1 << 20), __double2loint(v)) : ldexp(v, k);
+}
+// an FP32 integer below 2^22 in magnitude
+__device__ __forceinline__ int small_int(float v) { return __float_as_int(v + 12582912.f) - 0x4b400000; }
+
+// The digit pairs of one real product whose blocks leave the first Z weights
+// at zero.  A digit's registers take the next product's digit (na, nb; weights
+// from znext on) right after their last use here, so that the loads are in
+// flight under the multiplications that follow.
+template <int Z>
+__device__ __forceinline__ void multiply(float (&acc)[NW][4], uint4 (&a)[8], uint4 (&b)[4],
+                                         const uint4* __restrict__ na, const uint4* __restrict__ nb, int znext) {
+  constexpr int LAST = NW - 1 - Z;  // p + q <= LAST
+#pragma unroll
+  for (int p = 7; p >= 0; --p)
+    if (p > LAST && p + znext < NW) a[p] = na[32 * p];
+#pragma unroll
+  for (int q2 = 3; q2 >= 0; --q2)
+    if (2 * q2 > LAST && 2 * q2 + znext < NW) b[q2] = nb[32 * q2];
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    if (q <= LAST) {
+      const unsigned b0 = (q & 1) ? b[q >> 1].z : b[q >> 1].x, b1 = (q & 1) ? b[q >> 1].w : b[q >> 1].y;
+#pragma unroll
+      for (int p = 0; p < 8; ++p)
+        if (p + q <= LAST) mma16816(acc[p + q + Z], a[p], b0, b1);
+      if (((q & 1) || q == LAST) && (q & ~1) + znext < NW) b[q >> 1] = nb[32 * (q >> 1)];
+#pragma unroll
+      for (int p = 7; p >= 0; --p)
+        if (p <= LAST && (LAST - p < 7 ? LAST - p : 7) == q && p + znext < NW) a[p] = na[32 * p];
+    }
+  }
+}
+
+template <bool CPLX, bool ADAG, bool BDAG, int EPI>
+__global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_constant__ Args x) {
+  constexpr int NP = CPLX ? 2 : 1;  // real products per triple and warp; parts of a complex output
+  constexpr int WPI = 2 * NP;       // warps per item: 8-column halves x parts
+  const GemmArgs& g = x.g;
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int half = warp & 1;                      // output columns 8 half .. 8 half + 7
+  const int part = CPLX ? ((warp >> 1) & 1) : 0;  // 0: real part, 1: imaginary part
+  const int slot = warp / WPI;
+  const int64_t item = (int64_t)blockIdx.x * (WARPS / WPI) + slot;
+  if (item >= g.n_items) return;  // the warps of one item leave together
+
+  __shared__ double sC[WARPS / WPI][NE * NP];
+
+  // signs of the two real products of this part (op(A) = Ar + i sa Ai, op(B) = Br + i sb Bi):
+  //   real part:       Ar Br - sa sb Ai Bi;   imaginary part: sb Ar Bi + sa Ai Br
+  const bool neg0 = CPLX && part && BDAG;
+  const bool neg1 = CPLX && (part ? ADAG : (ADAG == BDAG));
+
+  float acc[NW][4], top[4];  // sums of each weight; the carry out of the first
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    top[r] = 0.f;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) acc[w][r] = 0.f;
+  }
+  // moves multiples of 256 up one weight (FP32 integers below 2^24: every operation is exact)
+  auto carry = [&] {
+    constexpr float MAGIC = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer
+#pragma unroll
+    for (int w = NW - 1; w >= 0; --w)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const float c = __fadd_rn(__fmaf_rn(acc[w][r], 1.f / 256.f, MAGIC), -MAGIC);
+        acc[w][r] = __fmaf_rn(c, -256.f, acc[w][r]);
+        if (w > 0) acc[w - 1][r] += c;
+        else top[r] += c;
+      }
+  };
+
+  const int64_t t0 = g.ptr[item], t1 = g.ptr[item + 1];
+  const int2* __restrict__ ab = g.ab;
+  const unsigned char* __restrict__ dA = x.dA + lane * 16;
+  const unsigned char* __restrict__ dB = x.dB + lane * 16 + half * (BLK / 2);
+  // digits to skip of a triple's blocks: bytes 0, 1: A's parts, bytes 2, 3: B's
+  auto leads = [&](int2 p) {
+    if constexpr (CPLX)
+      return (unsigned)reinterpret_cast<const unsigned short*>(x.lA)[p.x] |
+             (unsigned)reinterpret_cast<const unsigned short*>(x.lB)[p.y] << 16;
+    else
+      return (unsigned)x.lA[p.x] | (unsigned)x.lB[p.y] << 16;
+  };
+  auto lead_a = [&](unsigned z, int sub) { return (int)((z >> (8 * sub)) & 0xff); };
+  auto lead_b = [&](unsigned z, int sub) { return (int)((z >> (16 + 8 * (CPLX ? (sub ^ part) : 0))) & 0xff); };
+  if (t0 < t1) {
+    // triples t, t + 1 and t + 2 of the list; the digits to skip of the first two
+    int2 cur = ab[t0], nxt = t0 + 1 < t1 ? ab[t0 + 1] : cur, nxt2 = t0 + 2 < t1 ? ab[t0 + 2] : nxt;
+    unsigned zc = leads(cur), zn = leads(nxt);
+    uint4 a[8], b[4];
+    {
+      const uint4* pa = reinterpret_cast<const uint4*>(dA + (int64_t)cur.x * (BLK * NP));
+      const uint4* pb = reinterpret_cast<const uint4*>(dB + ((int64_t)cur.y * NP + part) * BLK);
+#pragma unroll
+      for (int p = 0; p < 8; ++p) a[p] = pa[32 * p];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) b[p] = pb[32 * p];
+    }
+    int since = 0;
+    for (int64_t t = t0; t < t1; ++t) {
+      const int2 nxt3 = t + 3 < t1 ? ab[t + 3] : nxt2;
+      const unsigned zn2 = leads(nxt2);
+#pragma unroll
+      for (int sub = 0; sub < NP; ++sub) {
+        // the blocks of the next real product (after the last one: this triple's again, unused)
+        const bool last = sub + 1 == NP;
+        const int2 nb = last ? nxt : cur;
+        const unsigned z = last ? zn : zc;
+        const int ns = CPLX ? (sub ^ 1) : 0;  // its part of A; of B: ns ^ part
+        const uint4* na = reinterpret_cast<const uint4*>(dA + ((int64_t)nb.x * NP + ns) * BLK);
+        const uint4* nbp = reinterpret_cast<const uint4*>(dB + ((int64_t)nb.y * NP + (CPLX ? (ns ^ part) : 0)) * BLK);
+        // weights below the first that can be non-zero, of this product and the next
+        const int zz = lead_a(zc, sub) + lead_b(zc, sub), znext = lead_a(z, ns) + lead_b(z, ns);
+        if (CPLX && (sub ? neg1 : neg0)) {
+#pragma unroll
+          for (int p = 0; p < 8; ++p) {
+            a[p].x ^= 0x80008000u;
+            a[p].y ^= 0x80008000u;
+            a[p].z ^= 0x80008000u;
+            a[p].w ^= 0x80008000u;
+          }
+        }
+        switch (zz) {
+          case 0: multiply<0>(acc, a, b, na, nbp, znext); break;
+          case 1: multiply<1>(acc, a, b, na, nbp, znext); break;
+          case 2: multiply<2>(acc, a, b, na, nbp, znext); break;
+          case 3: multiply<3>(acc, a, b, na, nbp, znext); break;
+          case 4: multiply<4>(acc, a, b, na, nbp, znext); break;
+          case 5: multiply<5>(acc, a, b, na, nbp, znext); break;
+          case 6: multiply<6>(acc, a, b, na, nbp, znext); break;
+          case 7: multiply<7>(acc, a, b, na, nbp, znext); break;
+          case 8: multiply<8>(acc, a, b, na, nbp, znext); break;
+          default: multiply<NW>(acc, a, b, na, nbp, znext); break;  // below every weight: nothing but the loads
+        }
+        if (++since == CARRY) {
+          carry();
+          since = 0;
+        }
+      }
+      cur = nxt;
+      nxt = nxt2;
+      nxt2 = nxt3;
+      zc = zn;
+      zn = zn2;
+    }
+    carry();
+  }
+
+  const int q = g.item_blk[item];
+  const int i = g.rowidx[q], j = g.colidx[q];
+  {
+    const int gr = lane >> 2, tc = lane & 3;
+#pragma unroll
+    for (int rr = 0; rr < 4; ++rr) {
+      const int r = gr + (rr >> 1) * 8, c = 8 * half + 2 * tc + (rr & 1);
+      if (r < BS && c < BS) {
+        // (hi 2^48 + lo) 256^6 2^-124: the integers enter FP64 as mantissas of 1.5 2^24 and
+        // 1.5 2^-24 (exact), and meet with one rounding
+        const int lo1 = (small_int(acc[3][rr]) * 256 + small_int(acc[4][rr])) * 256 + small_int(acc[5][rr]);
+        const int lo0 = (small_int(acc[6][rr]) * 256 + small_int(acc[7][rr])) * 256 + small_int(acc[8][rr]);
+        const int hi1 = __float2int_rn(top[rr]);
+        const int hi0 = (small_int(acc[0][rr]) * 256 + small_int(acc[1][rr])) * 256 + small_int(acc[2][rr]);
+        const long long lo = (long long)lo1 * (1 << 24) + lo0, hi = (long long)hi1 * (1 << 24) + hi0;
+        constexpr double MH = 0x1.8p24, ML = 0x1.8p-24;
+        const double vh = __longlong_as_double(__double_as_longlong(MH) + hi) - MH;
+        const double vl = __longlong_as_double(__double_as_longlong(ML) + lo) - ML;
+        sC[slot][(r * BS + c) * NP + part] = pow2_scaled(vh + vl, x.eA[i * 16 + r], x.eB[j * 16 + c]);
+      }
+    }
+  }
+  asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPI) : "memory");
+
+  using V = typename std::conditional<CPLX, double2, double>::type;
+  const V* val = reinterpret_cast<const V*>(sC[slot]);
+  const int el = lane + 32 * (warp % WPI);  // this thread's first element
+  constexpr int STEP = 32 * WPI;
+  V* __restrict__ C = static_cast<V*>(g.C);
+  if constexpr (EPI == EPI_STORE) {
+    for (int e = el; e < NE; e += STEP) C[(int64_t)q * NE + e] = val[e];
+  } else if constexpr (EPI == EPI_ADD) {
+    for (int e = el; e < NE; e += STEP) {
+      if constexpr (CPLX) {
+        const double2 o = C[(int64_t)q * NE + e];
+        C[(int64_t)q * NE + e] = make_double2(o.x + val[e].x, o.y + val[e].y);
+      } else {
+        C[(int64_t)q * NE + e] += val[e];
+      }
+    }
+  } else if constexpr (EPI == EPI_STORE_ACC) {
+    // real power T^n stored (unless C is null); coef * T^n added to complex U
+    double2* __restrict__ U = static_cast<double2*>(g.U);
+    const int uq = g.umap ? g.umap[q] : q;
+    for (int e = el; e < NE; e += STEP) {
+      if (C) C[(int64_t)q * NE + e] = val[e];
+      if (uq >= 0) {
+        double2 u = U[(int64_t)uq * NE + e];
+        if (g.coef_imag) u.y += g.coef * val[e];
+        else u.x += g.coef * val[e];
+        U[(int64_t)uq * NE + e] = u;
+      }
+    }
+  } else if constexpr (EPI == EPI_TWO_I) {
+    const int bi = g.bsize[i], bj = g.bsize[j];
+    double part_sum = 0.0;
+    for (int e = el; e < NE; e += STEP) {
+      const int r = e / BS, c = e - r * BS;
+      double re, im = 0.0;
+      if constexpr (CPLX) {
+        re = val[e].x;
+        im = val[e].y;
+      } else {
+        re = val[e];
+      }
+      const bool on = i == j && r == c;
+      const double dre = (on ? 1.0 : 0.0) - re;
+      if (r < bi && c < bj) part_sum += dre * dre + im * im;
+      if constexpr (CPLX) C[(int64_t)q * NE + e] = make_double2((on ? 2.0 : 0.0) - re, -im);
+      else C[(int64_t)q * NE + e] = (on ? 2.0 : 0.0) - re;
+    }
+    for (int off = 16; off > 0; off >>= 1) part_sum += __shfl_down_sync(0xffffffffu, part_sum, off);
+    __shared__ double partial[WARPS];
+    if (lane == 0) partial[warp] = part_sum;
+    asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPI) : "memory");
+    if (lane == 0 && warp % WPI == 0) {
+      double sum = 0.0;
+      for (int w = 0; w < WPI; ++w) sum += partial[warp + w];
+      g.red[item] = sum;
+    }
+  } else if constexpr (EPI == EPI_SANDWICH) {
+    // K'_ij for j >= i; mirror K'_ji = K'_ij^dagger; hermitian diagonal blocks
+    if (i != j) {
+      const int qt = g.tmap[q];
+      for (int e = el; e < NE; e += STEP) {
+        const int r = e / BS, c = e - r * BS;
+        C[(int64_t)q * NE + e] = val[e];
+        // the mirror, written in its own order: element (r,c) of block (j,i)
+        const double2 m = val[c * BS + r];
+        C[(int64_t)qt * NE + e] = make_double2(m.x, -m.y);
+      }
+    } else {
+      double herm = 0.0;
+      for (int e = el; e < NE; e += STEP) {
+        const int r = e / BS, c = e - r * BS;
+        const double2 v = val[e], tv = val[c * BS + r];
+        const double dr = v.x - tv.x, di = v.y + tv.y;  // K - K^dagger
+        herm = fmax(herm, sqrt(dr * dr + di * di));
+        C[(int64_t)q * NE + e] = make_double2(0.5 * (v.x + tv.x), 0.5 * (v.y - tv.y));
+      }
+      for (int off = 16; off > 0; off >>= 1) herm = fmax(herm, __shfl_xor_sync(0xffffffffu, herm, off));
+      if (lane == 0 && g.herm_max) atomicMax(g.herm_max, (unsigned long long)__double_as_longlong(herm));
+    }
+  }
+}
+
+template <bool CPLX, bool ADAG, bool BDAG, int EPI>
+static void launch(const Args& x, cudaStream_t st) {
+  const int64_t per = WARPS / (CPLX ? 4 : 2);
+  const int64_t grid = (x.g.n_items + per - 1) / per;
+  RT_REQUIRE(grid < (1ll << 31), RT_EINTERNAL, "grid too large");
+  k_gemm13_x64<CPLX, ADAG, BDAG, EPI><<<(unsigned)grid, WARPS * 32, 0, st>>>(x);
+  RT_CUDA_CHECK(cudaGetLastError());
+}
+
+}  // namespace x64
+
+size_t x64_block_bytes(bool cplx) { return (size_t)x64::BLK * (cplx ? 2 : 1); }
+
+void launch_split13(const void* vals, bool cplx, bool by_col, bool right, const Pattern& P, const X64Operand& out,
+                    cudaStream_t st) {
+  if (P.nnzb == 0 || P.n_atoms == 0) return;
+  if (cplx)
+    x64::k_split13<true><<<P.n_atoms, x64::SPLIT_WARPS * 32, 0, st>>>(static_cast<const double*>(vals), P.rowptr, P.tmap,
+                                                                      by_col, right, out.dig, out.lead, out.exps);
+  else
+    x64::k_split13<false><<<P.n_atoms, x64::SPLIT_WARPS * 32, 0, st>>>(static_cast<const double*>(vals), P.rowptr,
+                                                                       P.tmap, by_col, right, out.dig, out.lead, out.exps);
+  RT_CUDA_CHECK(cudaGetLastError());
+}
+
+void launch_gemm13_x64(bool cplx, bool a_dag, bool b_dag, Epilogue epi, const GemmArgs& g, const X64Operand& A,
+                       const X64Operand& B, cudaStream_t st) {
+  using namespace x64;
+  if (g.n_items == 0) return;
+  const Args x{g, A.dig, B.dig, A.lead, B.lead, A.exps, B.exps};
+  if (!cplx && !a_dag && !b_dag) {
+    if (epi == EPI_STORE) return launch<false, false, false, EPI_STORE>(x, st);
+    if (epi == EPI_STORE_ACC) return launch<false, false, false, EPI_STORE_ACC>(x, st);
+    if (epi == EPI_TWO_I) return launch<false, false, false, EPI_TWO_I>(x, st);
+    if (epi == EPI_ADD) return launch<false, false, false, EPI_ADD>(x, st);
+  } else if (cplx && !a_dag && !b_dag) {
+    if (epi == EPI_STORE) return launch<true, false, false, EPI_STORE>(x, st);
+    if (epi == EPI_TWO_I) return launch<true, false, false, EPI_TWO_I>(x, st);
+    if (epi == EPI_ADD) return launch<true, false, false, EPI_ADD>(x, st);
+  } else if (cplx && !a_dag && b_dag) {
+    if (epi == EPI_STORE) return launch<true, false, true, EPI_STORE>(x, st);
+    if (epi == EPI_SANDWICH) return launch<true, false, true, EPI_SANDWICH>(x, st);
+  } else if (cplx && a_dag && !b_dag) {
+    if (epi == EPI_STORE) return launch<true, true, false, EPI_STORE>(x, st);
+  }
+  throw Error{RT_EINTERNAL, "unsupported product variant"};
+}
+
+}  // namespace rt
