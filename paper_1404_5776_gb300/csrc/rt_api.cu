@@ -401,26 +401,14 @@ static void reserve_split(rt_ctx* c, const Sys& s, int64_t nnzb_a, int64_t nnzb_
   c->graph_dirty = true;  // a captured step holds the old addresses
 }
 
-// Gives the split operands back: in a mixed-precision EM, ETRS or M4 context only
-// the set-up has FP64 products, and at 10 A and 4096 atoms the two take 12.7 GB.
-static void release_split(rt_ctx* c) {
-  if (!c->xa.dig && !c->xb.dig) return;
-  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
-  for (X64Operand* x : {&c->xa, &c->xb}) {
-    for (void* p : {(void*)x->dig, (void*)x->lead, (void*)x->exps})
-      if (p) c->arena.put(p);
-    *x = X64Operand();
-  }
-  c->xa_bytes = c->xb_bytes = 0;
-  c->x_atoms = 0;
-}
-
 // keep_a: A is the operand of the product just before, unchanged since, so that its split stands
 static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cplx, bool ad, bool bd, Epilogue epi,
                  GemmArgs g, const Pattern* C, bool keep_a = false) {
   g = prepared(c, s, ti, fp32, cplx, epi, g, C);
   int B = s.B;
-  if (B == 13 && !fp32) {
+  if (B == 13 && c->p.precision == RT_FP64) {
+    // 13-function products of the FP64 mode: exact digit products on the tensor cores (6x the CUDA
+    // cores at every size measured, 64 to 512 atoms); the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
     if (!c->counting) reserve_split(c, s, ti.nnzb_a, ti.nnzb_b, cplx);
     run(
         c, cls, gemm_flops(ti, cplx), gemm_bytes(s, ti, cplx, fp32),
@@ -736,7 +724,7 @@ static void setup_system(rt_ctx* c, Sys& s, const rt_system& in) {
       s.planar = p.packed_fma != 0 && !p.tensor_cores;
     }
   }
-  if (s.B == 13 && (p.precision == RT_FP64 || p.prop == RT_PROP_CN)) {
+  if (s.B == 13 && p.precision == RT_FP64) {
     // the captured step holds FP64 products: their split operands are sized here
     int64_t most = 0;
     for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
@@ -2206,7 +2194,6 @@ rt_status rt_step(rt_ctx* c, int32_t n) {
     if (n == 0) return RT_OK;
     if (incremental(c))
       for (auto& sp : c->sys) prepare_reference(c, *sp);
-    if (c->p.precision == RT_FP32 && c->p.prop != RT_PROP_CN) release_split(c);
     build_groups(c);
     if (c->inject & RT_FAULT_WAIT_TIMEOUT_0) {
       // one step, launched directly, with a zero wait budget; the error word

@@ -6,7 +6,11 @@
 // triples: C_ij = sum_k op(A)_ik op(B)_kj for (i,j) in P_C, k ascending.  The
 // triple lists are built once (atoms are stationary).
 //
-// FP64 products of 13-function atoms run on the tensor cores (spgemm13_x64.cu).
+// FP64 products of 13-function atoms in an RT_FP64 context run on the tensor
+// cores (spgemm13_x64.cu); the FP64 set-up of the mixed modes stays here: a
+// mixed trajectory turns a last-bit change of its set-up into its FP32 noise
+// (4e-15 in K(0+) became 4e-10 of |K| after 60 steps at 512 atoms, 2e-9 in the
+// worst of 20 workloads), so these products keep their order of summation.
 //
 // Thread mapping: a group of LPB lanes owns one output block; each lane owns
 // EPL of its B*B elements and keeps them in registers.  Per triple the group
@@ -369,7 +373,9 @@ void launch_gemm(int B, bool fp32, bool cplx, bool a_dag, bool b_dag, Epilogue e
                         : dispatch_prec<1, double>(cplx, a_dag, b_dag, epi, g, st);
     case 4: return fp32 ? dispatch_prec<4, float>(cplx, a_dag, b_dag, epi, g, st)
                         : dispatch_prec<4, double>(cplx, a_dag, b_dag, epi, g, st);
-    case 13: throw Error{RT_EINTERNAL, "FP64 13-function products take split operands (launch_gemm13_x64)"};
+    case 13:
+      RT_REQUIRE(!fp32, RT_EINTERNAL, "FP32 13-function products use the padded block layout");
+      return dispatch_prec<13, double>(cplx, a_dag, b_dag, epi, g, st);
     default: throw Error{RT_EINVAL, "block size must pad to 1, 4 or 13"};
   }
 }
