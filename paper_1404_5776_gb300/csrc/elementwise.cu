@@ -2,6 +2,7 @@
 // identity/Taylor initialisation (eq. matrix_exp), the Crank-Nicolson operands,
 // the traces Tr(K S) and Tr(K D_j) (Sec. IV charge, Sec. II.B dipole), the
 // unitarity measure of eq. s_unit, and deterministic fixed-order reductions.
+#include <algorithm>
 #include <cmath>
 
 #include <cstring>
@@ -274,6 +275,11 @@ __global__ void k_sum_final(const double* __restrict__ part, int nb, double scal
   }
 }
 
+int trace_blocks(int64_t nnzb) {
+  const int64_t b = (nnzb + 4 * RED_T / 32 - 1) / (4 * RED_T / 32);  // four blocks (two upper ones) to a warp
+  return (int)std::min<int64_t>(std::max<int64_t>(b, 1), RED_MAXB);
+}
+
 int reduce_blocks(int64_t n) {
   int64_t b = (n + RED_T - 1) / RED_T;
   if (b < 1) b = 1;
@@ -292,55 +298,109 @@ void launch_sum(const double* v, int64_t n, double* part, double sqrt_div, doubl
 // diagonal blocks symmetrised) and every X is real symmetric, so
 //   Tr(K X) = sum_{i<j} 2 sum_ab Re K_ij[a,b] X_ji[b,a] + sum_i sum_ab Re K_ii[a,b] X_ii[b,a]
 // and Im Tr(K X) = 0 exactly; only the upper blocks are read.  X_ji comes
-// through kx_map (block (j,i) of X, or -1).  One warp per block (coalesced
-// reads of K), fixed block-to-warp assignment and fixed-order reductions: the
-// result does not depend on scheduling.
+// through kx_map (block (j,i) of X, or -1).  Fixed assignment of blocks to
+// lane groups and fixed-order reductions: the result does not depend on
+// scheduling.
+//
+// Bound by the FP64 pipe (four multiply-adds an element, two a clock and SM:
+// 31 us for the 27,400 upper blocks of 512 atoms x 13 at 8 A); a small system by
+// the length of the chain from the indices to the values, so the grid gives a
+// warp about two upper blocks as long as there are warps for it, and the next
+// block's indices load under the current block.  (One CTA per 256 blocks, as
+// before, left 16 CTAs at 64 atoms; both launches: 166 -> 29 us there, 163 -> 76 us
+// at 512 atoms.)
+struct TraceBlock {
+  int i, j, sq, dq;
+  bool on;
+};
+__device__ __forceinline__ TraceBlock trace_block(int64_t q, int64_t nnzb, const int32_t* __restrict__ rowidx,
+                                                  const int32_t* __restrict__ col, const int32_t* __restrict__ ks_map,
+                                                  const int32_t* __restrict__ kd_map) {
+  TraceBlock t{0, 0, -1, -1, q < nnzb};
+  if (t.on) t = {rowidx[q], col[q], ks_map[q], kd_map[q], true};
+  t.on = t.on && t.j >= t.i && (t.sq >= 0 || t.dq >= 0);
+  return t;
+}
+
 // One CTA's share (block index blk of nblk) of the trace sums of one K; its
-// 8 partials go to part[blk * 8 ..].
+// 8 partials go to part[blk * 8 ..].  BS: the block size where it is known to
+// the kernel (0: any), LPB lanes to a block.
+template <int BS, int LPB>
 __device__ __forceinline__ void traces_cta(const double2* __restrict__ K, int64_t nnzb,
+                                           const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
+                                           const int32_t* __restrict__ bsize, int Bany, const double* __restrict__ S,
+                                           const int32_t* __restrict__ ks_map, const double* __restrict__ Dx,
+                                           const double* __restrict__ Dy, const double* __restrict__ Dz,
+                                           const int32_t* __restrict__ kd_map, double* __restrict__ part, int blk,
+                                           int nblk) {
+  __shared__ double s[4][RED_T / 32];
+  constexpr int GROUPS = RED_T / LPB;
+  const int B = BS ? BS : Bany;
+  const int NE = B * B;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, gl = threadIdx.x % LPB;
+  double acc[4] = {0, 0, 0, 0};
+  const int64_t stride = (int64_t)nblk * GROUPS;
+  int64_t q = (int64_t)blk * GROUPS + threadIdx.x / LPB;
+  TraceBlock cur = trace_block(q, nnzb, rowidx, col, ks_map, kd_map);
+  for (; q < nnzb; q += stride) {
+    const TraceBlock next = trace_block(q + stride, nnzb, rowidx, col, ks_map, kd_map);
+    if (cur.on) {
+      const double w = (cur.i == cur.j) ? 1.0 : 2.0;
+      const int bi = bsize[cur.i], bj = bsize[cur.j];
+      const double2* k = K + q * NE;
+      const double* xs = S + (int64_t)cur.sq * NE;
+      const int64_t od = (int64_t)cur.dq * NE;
+#pragma unroll
+      for (int e0 = 0; e0 < (BS ? BS * BS : 169); e0 += LPB) {
+        const int e = e0 + gl;
+        if (!BS && e0 >= NE) break;
+        const int a = e / B, b = e - a * B;
+        if (e < NE && a < bi && b < bj) {
+          const double kr = w * k[e].x;
+          const int te = b * B + a;  // X_ji[b][a]
+          if (cur.sq >= 0) acc[0] += kr * xs[te];
+          if (cur.dq >= 0) {
+            acc[1] += kr * Dx[od + te];
+            acc[2] += kr * Dy[od + te];
+            acc[3] += kr * Dz[od + te];
+          }
+        }
+      }
+    }
+    cur = next;
+  }
+  // the four sums of the warp: halves and quarters of the lanes take two and then
+  // one of them on (6 additions a lane instead of 20: the FP64 pipe takes a warp's
+  // addition in 16 clocks)
+  {
+    const bool up = lane & 16, odd = lane & 8;
+    double a = up ? acc[2] : acc[0], b = up ? acc[3] : acc[1];
+    a += __shfl_xor_sync(0xffffffffu, up ? acc[0] : acc[2], 16);
+    b += __shfl_xor_sync(0xffffffffu, up ? acc[1] : acc[3], 16);
+    double v = odd ? b : a;
+    v += __shfl_xor_sync(0xffffffffu, odd ? a : b, 8);
+    for (int off = 4; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if ((lane & 7) == 0) s[(up ? 2 : 0) + (odd ? 1 : 0)][warp] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < 8) {  // Im Tr(K X) = 0 for hermitian K, symmetric X
+    double t = 0.0;
+    if (!(threadIdx.x & 1))
+      for (int w = 0; w < RED_T / 32; ++w) t += s[threadIdx.x >> 1][w];
+    part[blk * 8 + threadIdx.x] = t;
+  }
+}
+
+__device__ __forceinline__ void traces_any(const double2* __restrict__ K, int64_t nnzb,
                                            const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
                                            const int32_t* __restrict__ bsize, int B, const double* __restrict__ S,
                                            const int32_t* __restrict__ ks_map, const double* __restrict__ Dx,
                                            const double* __restrict__ Dy, const double* __restrict__ Dz,
                                            const int32_t* __restrict__ kd_map, double* __restrict__ part, int blk,
                                            int nblk) {
-  __shared__ double s[4][RED_T / 32];
-  double acc[4] = {0, 0, 0, 0};
-  const int NE = B * B;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t gw = (int64_t)blk * (RED_T / 32) + warp;
-  const int64_t nw = (int64_t)nblk * (RED_T / 32);
-  for (int64_t q = gw; q < nnzb; q += nw) {
-    int i = rowidx[q], j = col[q];
-    if (j < i) continue;
-    const double w = (i == j) ? 1.0 : 2.0;
-    int bi = bsize[i], bj = bsize[j];
-    int sq = ks_map[q], dq = kd_map[q];
-    const double2* k = K + q * NE;
-    for (int e = lane; e < bi * bj; e += 32) {
-      int a = e / bj, b = e - a * bj;
-      double kr = w * k[a * B + b].x;
-      int te = b * B + a;  // X_ji[b][a]
-      if (sq >= 0) acc[0] += kr * S[(int64_t)sq * NE + te];
-      if (dq >= 0) {
-        acc[1] += kr * Dx[(int64_t)dq * NE + te];
-        acc[2] += kr * Dy[(int64_t)dq * NE + te];
-        acc[3] += kr * Dz[(int64_t)dq * NE + te];
-      }
-    }
-  }
-  for (int c = 0; c < 4; ++c)
-    for (int off = 16; off > 0; off >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], off);
-  if (lane == 0)
-    for (int c = 0; c < 4; ++c) s[c][warp] = acc[c];
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int c = 0; c < 4; ++c) {
-      double t = 0.0;
-      for (int w = 0; w < RED_T / 32; ++w) t += s[c][w];
-      part[blk * 8 + 2 * c] = t;
-      part[blk * 8 + 2 * c + 1] = 0.0;  // Im Tr(K X) = 0 for hermitian K, symmetric X
-    }
+  if (B == 13) traces_cta<13, 32>(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part, blk, nblk);
+  else if (B == 4) traces_cta<4, 16>(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part, blk, nblk);
+  else traces_cta<0, 32>(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part, blk, nblk);
 }
 
 __global__ void k_traces(const double2* __restrict__ K, int64_t nnzb, const int32_t* __restrict__ rowidx,
@@ -348,14 +408,14 @@ __global__ void k_traces(const double2* __restrict__ K, int64_t nnzb, const int3
                          const double* __restrict__ S, const int32_t* __restrict__ ks_map,
                          const double* __restrict__ Dx, const double* __restrict__ Dy, const double* __restrict__ Dz,
                          const int32_t* __restrict__ kd_map, double* __restrict__ part) {
-  traces_cta(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part, blockIdx.x, gridDim.x);
+  traces_any(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part, blockIdx.x, gridDim.x);
 }
 
 // The same for every (system, kick) pair of a table: pair blockIdx.y, its
 // partials at part[pair * gridDim.x * 8 ..].
 __global__ void k_traces_grouped(const TracePair* __restrict__ tab, double* __restrict__ part) {
   const TracePair& t = tab[blockIdx.y];
-  traces_cta(t.K, t.nnzb, t.rowidx, t.col, t.bsize, t.B, t.S, t.ks_map, t.Dx, t.Dy, t.Dz, t.kd_map,
+  traces_any(t.K, t.nnzb, t.rowidx, t.col, t.bsize, t.B, t.S, t.ks_map, t.Dx, t.Dy, t.Dz, t.kd_map,
              part + (int64_t)blockIdx.y * gridDim.x * 8, blockIdx.x, gridDim.x);
 }
 
@@ -364,17 +424,18 @@ __device__ __forceinline__ void traces_final_cta(const double* __restrict__ part
                                                  int herm_slot, double* __restrict__ ring, int capacity, int n_slots,
                                                  int slot_index, const double* __restrict__ ref,
                                                  double* __restrict__ out) {
-  __shared__ double s[8][RED_T];
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int i = threadIdx.x; i < nb; i += RED_T)
-    for (int c = 0; c < 8; ++c) acc[c] += part[i * 8 + c];
-  for (int c = 0; c < 8; ++c) s[c][threadIdx.x] = acc[c];
+  // thread (component, one of RED_T/8 strides over the partials); fixed order
+  __shared__ double s[8][RED_T / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double acc = 0.0;
+  for (int i = threadIdx.x >> 3; i < nb; i += RED_T / 8) acc += part[i * 8 + (threadIdx.x & 7)];
+  acc += __shfl_down_sync(0xffffffffu, acc, 16);
+  acc += __shfl_down_sync(0xffffffffu, acc, 8);
+  if (lane < 8) s[lane][warp] = acc;
   __syncthreads();
-  for (int off = RED_T / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off)
-      for (int c = 0; c < 8; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + off];
-    __syncthreads();
-  }
+  if (threadIdx.x < 8)
+    for (int w = 1; w < RED_T / 32; ++w) s[threadIdx.x][0] += s[threadIdx.x][w];
+  __syncthreads();
   if (threadIdx.x == 0 && ref)  // incremental form: traces of K_ref + dK
     for (int c = 0; c < 8; ++c) s[c][0] += ref[c];
   if (threadIdx.x == 0 && out) {  // plain output (reference traces)
@@ -420,7 +481,7 @@ void launch_traces(const double2* K, int64_t nnzb, const int32_t* rowidx, const 
                    const double* Dz, const int32_t* kd_map, double* part, const DevState* st, int herm_slot,
                    double* ring, int capacity, int n_slots, int slot_index, cudaStream_t s, const double* ref,
                    double* out) {
-  int nb = reduce_blocks(nnzb);
+  int nb = trace_blocks(nnzb);
   k_traces<<<nb, RED_T, 0, s>>>(K, nnzb, rowidx, col, bsize, B, S, ks_map, Dx, Dy, Dz, kd_map, part);
   k_traces_final<<<1, RED_T, 0, s>>>(part, nb, st, herm_slot, ring, capacity, n_slots, slot_index, ref, out);
   RT_CUDA_CHECK(cudaGetLastError());

@@ -101,7 +101,7 @@ RT_API rt_status rt_traces_noalloc(const double* K, int64_t nnzb, const int32_t*
   if (nnzb < 0 || B < 1 || B > 13) return fail(RT_EINVAL, "nnzb must be >= 0 and B in 1..13");
   int nb = n_ctas;
   if (nb == 0) {
-    int64_t want = (nnzb + kThreads - 1) / kThreads;
+    int64_t want = (nnzb + 4 * kThreads / 32 - 1) / (4 * kThreads / 32);  // four blocks (two upper ones) to a warp
     nb = (int)(want < 1 ? 1 : (want > kMaxCtas ? kMaxCtas : want));
   }
   if (nb < 1 || nb > kMaxCtas)

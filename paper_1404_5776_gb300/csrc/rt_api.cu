@@ -1508,7 +1508,7 @@ static void build_groups(rt_ctx* c) {
         c->tbytes += 16.0 * nvals(s, s.pK) + 8.0 * 4 * nvals(s, s.pH);
       }
     }
-    c->tnb = reduce_blocks(max_nnzb);
+    c->tnb = trace_blocks(max_nnzb);
     c->d_tpairs = c->arena.get_n<TracePair>(tp.size());
     c->tpart = c->arena.get_n<double>((size_t)tp.size() * c->tnb * 8);
     RT_CUDA_CHECK(

@@ -42,6 +42,7 @@ void launch_restrict(const double* src, double* dst, const int32_t* map, int64_t
 void launch_cn_operands(const double* S, const int32_t* a_to_s, const double* H, const int32_t* a_to_h, double c,
                         double2* A, double2* Bm, int64_t nnzb_a, int B, cudaStream_t st);
 int reduce_blocks(int64_t n);
+int trace_blocks(int64_t nnzb);  // CTAs of the trace sums of nnzb blocks
 void launch_sum(const double* v, int64_t n, double* part, double sqrt_div, double* out, double* out2,
                 cudaStream_t st);
 void launch_traces(const double2* K, int64_t nnzb, const int32_t* rowidx, const int32_t* col, const int32_t* bsize,
@@ -62,7 +63,7 @@ struct TracePair {
   int herm_slot, slot_index;
   const double* ref;
 };
-// launch_traces for every pair of a device table in two launches: nb CTAs per pair (reduce_blocks of the
+// launch_traces for every pair of a device table in two launches: nb CTAs per pair (trace_blocks of the
 // largest pair), partials in part[n_pairs][nb][8], one observables record per pair
 void launch_traces_grouped(const TracePair* tab, int n_pairs, int nb, double* part, const DevState* st, double* ring,
                            int capacity, int n_slots, cudaStream_t s);
