@@ -1077,6 +1077,7 @@ __global__ void __launch_bounds__(POLY_WARPS * 32) k_field_poly(PolyTerms V, int
   __shared__ float2 tiles[POLY_WARPS][13 * 13];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double E = s->E[which];
+  if (E == 0.0) deg = 0;  // U(0) = V_0: without a field one coefficient of deg + 1 is read
   const float Ef = (float)E;
   const int64_t step = s->step;
   const int NE = B * B;

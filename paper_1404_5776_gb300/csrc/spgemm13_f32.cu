@@ -442,17 +442,18 @@ __device__ __forceinline__ int c32_item(const GemmArgs& g, int64_t item, float2*
       // coefficient by coefficient, so that the lane's loads of one B_p are
       // in flight together
       const double E = *g.poly_E;
+      const int deg = E == 0.0 ? 0 : g.rdeg;  // without a field R(0) = B_0: one coefficient is read
       constexpr int HALF = (EPT + 1) / 2;  // elements per pass (register budget)
 #pragma unroll
       for (int k0 = 0; k0 < EPT; k0 += HALF) {
         double2 rv[HALF];
-        const double2* __restrict__ top = g.rpoly[g.rdeg];
+        const double2* __restrict__ top = g.rpoly[deg];
 #pragma unroll
         for (int k = 0; k < HALF; ++k) {
           const int e = lane + 32 * (k0 + k);
           rv[k] = (k0 + k < EPT && e < NE) ? top[(int64_t)q * NE + e] : make_double2(0.0, 0.0);
         }
-        for (int p = g.rdeg - 1; p >= 0; --p) {
+        for (int p = deg - 1; p >= 0; --p) {
           const double2* __restrict__ cp = g.rpoly[p];
 #pragma unroll
           for (int k = 0; k < HALF; ++k) {

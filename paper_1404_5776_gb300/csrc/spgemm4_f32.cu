@@ -157,6 +157,7 @@ __device__ __forceinline__ void g4_item(const GemmArgs& g, int64_t item) {
       const double2* __restrict__ R = g.base2 ? static_cast<const double2*>(g.base2) + (int64_t)q * NE : nullptr;
       // or R(E) = sum_p E^p B_p at this step's field, by Horner here
       const double E = g.rpoly ? *g.poly_E : 0.0;
+      const int deg = E == 0.0 ? 0 : g.rdeg;  // R(0) = B_0
 #pragma unroll
       for (int r = 0; r < 4; ++r)
 #pragma unroll
@@ -167,8 +168,8 @@ __device__ __forceinline__ void g4_item(const GemmArgs& g, int64_t item) {
             kv = make_double2(kv.x + R[e].x, kv.y + R[e].y);
           } else if (g.rpoly) {
             const int64_t idx = (int64_t)q * NE + e;
-            double2 rv = g.rpoly[g.rdeg][idx];
-            for (int p = g.rdeg - 1; p >= 0; --p) {
+            double2 rv = g.rpoly[deg][idx];
+            for (int p = deg - 1; p >= 0; --p) {
               const double2 cp = g.rpoly[p][idx];
               rv = make_double2(fma(rv.x, E, cp.x), fma(rv.y, E, cp.y));
             }
