@@ -307,7 +307,7 @@ class RT:
     def matrix(self, sys: int, which: int, kick: int = 0) -> np.ndarray:
         n = ctypes.c_int64()
         self._c(self.lib.rt_matrix_size(self.ctx, sys, which, ctypes.byref(n)))
-        out = np.zeros(max(n.value, 2), dtype=np.float64)
+        out = np.empty(max(n.value, 2), dtype=np.float64)  # written whole
         self._c(self.lib.rt_get_matrix(self.ctx, sys, kick, which, _p(out), n.value))
         return out[:n.value].view(np.complex128)
 
@@ -341,7 +341,7 @@ class RT:
 
     def observables(self, sys: int = 0, kick: int = 0, max_steps: Optional[int] = None) -> np.ndarray:
         cap = max_steps or self.params.obs_capacity
-        out = np.zeros((cap, RT_NOBS), dtype=np.float64)
+        out = np.empty((cap, RT_NOBS), dtype=np.float64)
         n = ctypes.c_int32()
         st = self.lib.rt_observables(self.ctx, sys, kick, _p(out), cap, ctypes.byref(n))
         if st not in (RT_OK, RT_ENUMERIC):
@@ -391,7 +391,10 @@ class RT:
         return buf.raw
 
     def set_state(self, data: bytes):
-        buf = ctypes.create_string_buffer(data, len(data))
+        if isinstance(data, bytes):  # read in place
+            self._c(self.lib.rt_set_state(self.ctx, ctypes.c_char_p(data), len(data)))
+            return
+        buf = ctypes.create_string_buffer(bytes(data), len(data))
         self._c(self.lib.rt_set_state(self.ctx, buf, len(data)))
 
     def synchronize(self):

@@ -19,6 +19,7 @@
 #include <limits>
 #include <map>
 #include <memory>
+#include <thread>
 #include <tuple>
 
 #include "rt_elementwise.cuh"
@@ -68,6 +69,7 @@ struct Sys {
           *pM = nullptr, *pA = nullptr, *pW = nullptr;
   std::map<double, std::unique_ptr<Pattern>> pcache;
   std::unique_ptr<Pattern> pS_given, pH_given;
+  std::map<const Pattern*, int64_t*> true_off;  // padded systems: first true element of each block (device)
   std::map<TripleKey, std::unique_ptr<TripleInfo>> tcache;
   // FP64 values (padded blocks)
   double *S = nullptr, *H0 = nullptr, *D[3] = {nullptr, nullptr, nullptr}, *Hm = nullptr;
@@ -125,6 +127,10 @@ struct Sys {
   std::string sinv_status;
 };
 
+// Host copies: threads that share one large pageable copy, and the pinned piece of each
+constexpr int IO_THREADS = 8;
+constexpr size_t IO_PIECE = size_t(2) << 20;
+
 // Grouped products of the reference split (one launch per product and block
 // size across all (system, kick) pairs) and their launch shapes
 constexpr int RT_N_STAGES = 4;  // 13-function M, 13-function K', 4-function M, 4-function K'
@@ -165,6 +171,9 @@ struct rt_ctx {
   rt::X64Operand xa, xb;
   size_t xa_bytes = 0, xb_bytes = 0;
   int x_atoms = 0;
+  // pinned staging of host copies to and from pageable memory (made by the first large one)
+  void* stage = nullptr;
+  cudaEvent_t stage_ev[rt::IO_THREADS] = {};
   void* zero32 = nullptr;  // one zero FP32 complex block (padded layout)
   int* d_err = nullptr;    // device error word of bounded waits
   long long wait_ns = 2000000000ll;  // budget of one bounded device wait
@@ -1212,9 +1221,9 @@ static void observe(rt_ctx* c, Sys& s, int kick, int slot) {
 // K = K_ref + dK for the kicks whose K is stale.  keep = false hands K back
 // as the authoritative density (the next step forms dK = K - K_ref again);
 // a read (keep = true) leaves dK in place, so the run continues unchanged.
-static void materialize(rt_ctx* c, Sys& s, bool keep = false) {
+static void materialize(rt_ctx* c, Sys& s, bool keep = false, int only = -1) {
   for (size_t k = 0; k < s.dk_fresh.size(); ++k) {
-    if (!s.dk_fresh[k]) continue;
+    if (!s.dk_fresh[k] || (only >= 0 && (int)k != only)) continue;
     launch_zaxpy(s.K[k], s.Kref, s.dK[k], 1.0, (int64_t)nvals(s, s.pK), c->ws);
     if (!keep) s.dk_fresh[k] = 0;
   }
@@ -1317,9 +1326,10 @@ static void reference_split_propagator(rt_ctx* c, Sys& s) {
     PolyTerms32 T;
     memset(&T, 0, sizeof(T));
     const bool tail = (int)s.V32.size() == deg + 1;
+    const int read = c->field.kind == RT_FIELD_NONE ? 0 : deg;  // without a field V_0 alone is read
     for (int m = 1; m <= deg && tail; ++m) T.v[m] = s.V32[m];
     // read V_0 (FP64) and V_1..V_deg (FP32 tail), write dU and dU^dagger
-    run(c, PC_POLY, 0, 16.0 * nU + (tail ? 8.0 : 16.0) * nU * deg + 16.0 * nU, [&] {
+    run(c, PC_POLY, 0, 16.0 * nU + (tail ? 8.0 : 16.0) * nU * read + 16.0 * nU, [&] {
       launch_field_poly(V, deg, c->dstate, 0, nullptr, s.dUr, s.dUHr, s.pU->nnzb, s.pU->rowidx, s.pU->col, s.B,
                         c->ws, true, s.planar, tail ? &T : nullptr);
     });
@@ -1809,6 +1819,82 @@ static Pattern* pattern_by_id(Sys& s, int which) {
   }
 }
 
+// Copies between the device and caller memory and waits.  A pinned buffer takes
+// one DMA.  Pageable memory of some size goes through pinned pieces, one per
+// thread: the host side of such a copy is bound by one core's memcpy and by the
+// first touch of the caller's pages, which the threads share (K of 512 atoms x 13
+// at 8 A, 148 MB into a new array: 25 -> 8 ms with the rest of the read).
+static void copy_host(rt_ctx* c, void* dst, const void* src, size_t bytes, bool to_host) {
+  const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
+  cudaPointerAttributes at{};
+  const bool known = cudaPointerGetAttributes(&at, to_host ? dst : src) == cudaSuccess;
+  if (!known) cudaGetLastError();
+  const bool pinned = known && at.type != cudaMemoryTypeUnregistered;
+  if (pinned || bytes < 2 * IO_PIECE) {
+    if (bytes) RT_CUDA_CHECK(cudaMemcpyAsync(dst, src, bytes, kind, c->ws));
+    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+    return;
+  }
+  if (!c->stage) {
+    for (cudaEvent_t& e : c->stage_ev)
+      if (!e) RT_CUDA_CHECK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    RT_CUDA_CHECK(cudaMallocHost(&c->stage, IO_THREADS * IO_PIECE));
+  }
+  int dev = 0;
+  RT_CUDA_CHECK(cudaGetDevice(&dev));
+  const size_t pieces = (bytes + IO_PIECE - 1) / IO_PIECE;
+  const int n = (int)std::min<size_t>(IO_THREADS, pieces);
+  cudaError_t errs[IO_THREADS] = {};
+  // thread w moves the pieces w, w + n, ... through its own buffer; the copies of
+  // all threads follow one another on the context's stream
+  auto work = [&](int w) {
+    cudaError_t e = cudaSetDevice(dev);
+    char* buf = static_cast<char*>(c->stage) + (size_t)w * IO_PIECE;
+    for (size_t k = w; k < pieces && e == cudaSuccess; k += n) {
+      const size_t off = k * IO_PIECE, nb = std::min(IO_PIECE, bytes - off);
+      char* d = static_cast<char*>(dst) + off;
+      const char* s = static_cast<const char*>(src) + off;
+      if (!to_host) memcpy(buf, s, nb);
+      e = cudaMemcpyAsync(to_host ? buf : d, to_host ? s : buf, nb, kind, c->ws);
+      if (e == cudaSuccess) e = cudaEventRecord(c->stage_ev[w], c->ws);
+      if (e == cudaSuccess) e = cudaEventSynchronize(c->stage_ev[w]);
+      if (e == cudaSuccess && to_host) memcpy(d, buf, nb);
+    }
+    errs[w] = e;
+  };
+  std::vector<std::thread> pool;
+  int started = 1;
+  try {
+    for (; started < n; ++started) pool.emplace_back(work, started);
+  } catch (...) {  // no more threads to be had: this one takes their pieces
+  }
+  work(0);
+  for (std::thread& t : pool) t.join();
+  for (int w = started; w < n; ++w) work(w);
+  for (int w = 0; w < n; ++w) RT_CUDA_CHECK(errs[w]);
+  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+}
+
+// First true element of each block of P in the caller's layout (padded systems; device)
+static const int64_t* true_offsets(rt_ctx* c, Sys& s, const Pattern* P) {
+  auto it = s.true_off.find(P);
+  if (it != s.true_off.end()) return it->second;
+  std::vector<int64_t> off(P->nnzb);
+  int64_t n = 0;
+  for (int i = 0; i < s.n_atoms; ++i)
+    for (int q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
+      off[q] = n;
+      n += (int64_t)s.bsize[i] * s.bsize[P->h_col[q]];
+    }
+  int64_t* d = c->arena.get_n<int64_t>(off.size());
+  if (!off.empty())
+    RT_CUDA_CHECK(cudaMemcpyAsync(d, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice, c->ws));
+  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+  s.true_off[P] = d;
+  return d;
+}
+static bool padded(const Sys& s) { return s.n_true != (int64_t)s.n_atoms * s.B; }
+
 // (pattern, device values, complex?) of a readable matrix
 static void matrix_by_id(rt_ctx* c, Sys& s, int kick, int which, Pattern** P, const void** v, bool* cplx) {
   *cplx = false;
@@ -2047,30 +2133,19 @@ rt_status rt_set_density(rt_ctx* c, int32_t sys, int32_t kick, const double* h) 
     // K replaced: it is the density again; the reference split keeps K_ref and
     // carries the new K as dK = K - K_ref from the next step
     if (!s.dk_fresh.empty()) s.dk_fresh[kick] = 0;
-    if (s.n_true == (int64_t)s.n_atoms * B) {
+    if (!padded(s)) {
       // no padded atoms: the caller's layout is the device layout; copy directly
       // (a DMA at full speed when the caller's buffer is pinned)
-      RT_CUDA_CHECK(cudaMemcpyAsync(s.K[kick], h, sizeof(double2) * nvals(s, s.pK), cudaMemcpyHostToDevice, c->ws));
       reset_time(c);
-      RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+      copy_host(c, s.K[kick], h, sizeof(double2) * nvals(s, s.pK), false);
       return RT_OK;
     }
-    std::vector<double> buf(2 * (size_t)P.nnzb * B * B, 0.0);
-    size_t o = 0;
-    for (int i = 0; i < s.n_atoms; ++i)
-      for (int q = P.h_rowptr[i]; q < P.h_rowptr[i + 1]; ++q) {
-        int j = P.h_col[q];
-        int bi = s.bsize[i], bj = s.bsize[j];
-        double* blk = buf.data() + 2 * (size_t)q * B * B;
-        for (int a = 0; a < bi; ++a)
-          for (int b = 0; b < bj; ++b) {
-            blk[2 * (a * B + b)] = h[2 * (o + (size_t)a * bj + b)];
-            blk[2 * (a * B + b) + 1] = h[2 * (o + (size_t)a * bj + b) + 1];
-          }
-        o += (size_t)bi * bj;
-      }
-    RT_CUDA_CHECK(cudaMemcpyAsync(s.K[kick], buf.data(), sizeof(double) * buf.size(), cudaMemcpyHostToDevice, c->ws));
+    const int64_t n = true_elems(s, &P);
+    Scratch tmp(c);
+    double2* compact = tmp.get_n<double2>(n);
     reset_time(c);
+    copy_host(c, compact, h, sizeof(double2) * n, false);
+    launch_unpack_true(compact, true_offsets(c, s, &P), P.nnzb, P.rowidx, P.col, s.d_bsize, B, s.K[kick], c->ws);
     RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
     return RT_OK;
   });
@@ -2256,14 +2331,20 @@ rt_status rt_observables(rt_ctx* c, int32_t sys, int32_t kick, double* out, int3
     int64_t cap = c->p.obs_capacity;
     int64_t first = std::max(c->read_upto[slot], c->host_step - cap);
     int64_t cnt = std::min<int64_t>(c->host_step - first, max_steps);
-    std::vector<double> ring((size_t)cap * c->n_slots * RT_NOBS);
-    RT_CUDA_CHECK(cudaMemcpyAsync(ring.data(), c->ring, sizeof(double) * ring.size(), cudaMemcpyDeviceToHost, c->ws));
+    // the records of the steps asked for (one or two runs of the ring)
+    const size_t row = (size_t)c->n_slots * RT_NOBS;
+    std::vector<double> recs((size_t)std::max<int64_t>(cnt, 0) * row);
+    for (int64_t k = 0; k < cnt;) {
+      const int64_t r = (first + k) % cap, m = std::min(cnt - k, cap - r);
+      RT_CUDA_CHECK(cudaMemcpyAsync(recs.data() + k * row, c->ring + r * row, sizeof(double) * m * row,
+                                    cudaMemcpyDeviceToHost, c->ws));
+      k += m;
+    }
     RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
     check_device_error(c);
     bool bad = false;
     for (int64_t k = 0; k < cnt; ++k) {
-      int64_t r = (first + k) % cap;
-      const double* rec = ring.data() + (r * c->n_slots + slot) * RT_NOBS;
+      const double* rec = recs.data() + k * row + (size_t)slot * RT_NOBS;
       for (int v = 0; v < RT_NOBS; ++v) {
         out[k * RT_NOBS + v] = rec[v];
         if (!std::isfinite(rec[v])) bad = true;
@@ -2325,7 +2406,7 @@ rt_status rt_get_matrix(rt_ctx* c, int32_t sys, int32_t kick, int32_t which, dou
     Pattern* P;
     const void* v;
     bool cplx;
-    if (which == RT_MAT_K) materialize(c, s, true);
+    if (which == RT_MAT_K) materialize(c, s, true, kick);
     if (which == RT_MAT_U) refresh_u64(c, s);
     if (which == RT_MAT_U && s.duf_current)
       launch_u_from_delta(s.dUf, s.U, s.pU->nnzb, s.pU->rowidx, s.pU->col, s.B, c->ws);  // U = I + (U - I)
@@ -2333,24 +2414,15 @@ rt_status rt_get_matrix(rt_ctx* c, int32_t sys, int32_t kick, int32_t which, dou
     RT_REQUIRE(vals, RT_EINVAL, "NULL output");
     int64_t need = 2 * true_elems(s, P);
     RT_REQUIRE(capacity >= need, RT_EINVAL, "output buffer too small");
-    const int B = s.B;
-    size_t nv = (size_t)P->nnzb * B * B * (cplx ? 2 : 1);
-    std::vector<double> buf(nv);
-    if (nv) RT_CUDA_CHECK(cudaMemcpyAsync(buf.data(), v, sizeof(double) * nv, cudaMemcpyDeviceToHost, c->ws));
-    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
-    size_t o = 0;
-    for (int i = 0; i < s.n_atoms; ++i)
-      for (int q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
-        int j = P->h_col[q];
-        int bi = s.bsize[i], bj = s.bsize[j];
-        for (int a = 0; a < bi; ++a)
-          for (int b = 0; b < bj; ++b) {
-            size_t e = (size_t)q * B * B + a * B + b;
-            vals[2 * o] = cplx ? buf[2 * e] : buf[e];
-            vals[2 * o + 1] = cplx ? buf[2 * e + 1] : 0.0;
-            ++o;
-          }
-      }
+    if (cplx && !padded(s)) {  // the device layout is the caller's
+      copy_host(c, vals, v, sizeof(double) * need, true);
+      return RT_OK;
+    }
+    Scratch tmp(c);
+    double2* compact = tmp.get_n<double2>(need / 2);
+    launch_pack_true(v, cplx, padded(s) ? true_offsets(c, s, P) : nullptr, P->nnzb, P->rowidx, P->col, s.d_bsize, s.B,
+                     compact, c->ws);
+    copy_host(c, vals, compact, sizeof(double) * need, true);
     return RT_OK;
   });
 }
@@ -2470,14 +2542,14 @@ rt_status rt_get_state(rt_ctx* c, void* buf, size_t* bytes) {
       Sys& s = *sp;
       for (double2* K : s.K) {
         size_t nb = sizeof(double2) * nvals(s, s.pK);
-        RT_CUDA_CHECK(cudaMemcpyAsync(o, K, nb, cudaMemcpyDeviceToHost, c->ws));
+        copy_host(c, o, K, nb, true);
         o += nb;
       }
       size_t nu = sizeof(double2) * nvals(s, s.pU);
-      RT_CUDA_CHECK(cudaMemcpyAsync(o, s.U, nu, cudaMemcpyDeviceToHost, c->ws));
+      copy_host(c, o, s.U, nu, true);
       o += nu;
       if (s.X) {
-        RT_CUDA_CHECK(cudaMemcpyAsync(o, s.X, nu, cudaMemcpyDeviceToHost, c->ws));
+        copy_host(c, o, s.X, nu, true);
         o += nu;
       }
     }
@@ -2529,14 +2601,14 @@ rt_status rt_set_state(rt_ctx* c, const void* buf, size_t bytes) {
       if (!c->p.full_step) s.r_ready = false;                  // a constant U's R follows the restored U
       for (double2* K : s.K) {
         size_t nb = sizeof(double2) * nvals(s, s.pK);
-        RT_CUDA_CHECK(cudaMemcpyAsync(K, o, nb, cudaMemcpyHostToDevice, c->ws));
+        copy_host(c, K, o, nb, false);
         o += nb;
       }
       size_t nu = sizeof(double2) * nvals(s, s.pU);
-      RT_CUDA_CHECK(cudaMemcpyAsync(s.U, o, nu, cudaMemcpyHostToDevice, c->ws));
+      copy_host(c, s.U, o, nu, false);
       o += nu;
       if (s.X) {
-        RT_CUDA_CHECK(cudaMemcpyAsync(s.X, o, nu, cudaMemcpyHostToDevice, c->ws));
+        copy_host(c, s.X, o, nu, false);
         o += nu;
       }
       if (c->p.precision == RT_FP32 && s.dUf) {
@@ -2638,6 +2710,9 @@ void rt_destroy(rt_ctx* c) {
     cudaEventDestroy(e.second);
   }
   c->arena.release_all();
+  if (c->stage) cudaFreeHost(c->stage);
+  for (cudaEvent_t e : c->stage_ev)
+    if (e) cudaEventDestroy(e);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ws) cudaStreamDestroy(c->ws);
