@@ -596,4 +596,39 @@ int64_t triple_true_macs(const Triples& T, const Pattern& A, bool a_dag, const P
   return (int64_t)h;
 }
 
+// Host pass over the rows of one group at a time: the groups that its atoms
+// reach, ascending, and the blocks of each.
+void build_quads(QuadPattern& Q, const Pattern& P, Arena& arena, cudaStream_t st) {
+  const int n = P.n_atoms, m = (n + 3) / 4;
+  std::vector<int32_t> rowptr(m + 1, 0), col, map, seen(m, -1), cols;
+  for (int I = 0; I < m; ++I) {
+    cols.clear();
+    const int i1 = std::min(n, 4 * I + 4);
+    for (int i = 4 * I; i < i1; ++i)
+      for (int q = P.h_rowptr[i]; q < P.h_rowptr[i + 1]; ++q) {
+        const int J = P.h_col[q] >> 2;
+        if (seen[J] >= 0) continue;
+        seen[J] = 0;
+        cols.push_back(J);
+      }
+    std::sort(cols.begin(), cols.end());
+    const size_t base = col.size();
+    for (size_t k = 0; k < cols.size(); ++k) seen[cols[k]] = (int32_t)k;
+    col.insert(col.end(), cols.begin(), cols.end());
+    map.resize(col.size() * 16, -1);
+    for (int i = 4 * I; i < i1; ++i)
+      for (int q = P.h_rowptr[i]; q < P.h_rowptr[i + 1]; ++q) {
+        const int j = P.h_col[q];
+        map[(base + seen[j >> 2]) * 16 + (i & 3) * 4 + (j & 3)] = q;
+      }
+    for (int J : cols) seen[J] = -1;
+    rowptr[I + 1] = (int32_t)col.size();
+  }
+  upload_pattern(Q.P, m, rowptr.data(), col.data(), P.radius, arena, st);
+  Q.map = arena.get_n<int32_t>(map.size());
+  if (!map.empty())
+    RT_CUDA_CHECK(cudaMemcpyAsync(Q.map, map.data(), sizeof(int32_t) * map.size(), cudaMemcpyHostToDevice, st));
+  RT_CUDA_CHECK(cudaStreamSynchronize(st));
+}
+
 }  // namespace rt

@@ -48,6 +48,11 @@ struct TripleKey {
 struct TripleInfo {
   const Pattern *pa = nullptr, *pb = nullptr;  // the operands' patterns
   Triples t;
+  // FP64 4-function products as quads (16 x 16 blocks of four consecutive atoms): the quads'
+  // list and patterns; taken where `quads`
+  Triples qt;
+  const QuadPattern *qa = nullptr, *qb = nullptr, *qc = nullptr;
+  bool quads = false;
   TileList tiles;  // row tiles for the tensor-core kernel (built for the sandwich's FP32 13-function products)
   int64_t true_macs = 0;
   int64_t nnzb_a = 0, nnzb_b = 0;
@@ -71,6 +76,7 @@ struct Sys {
   std::unique_ptr<Pattern> pS_given, pH_given;
   std::map<const Pattern*, int64_t*> true_off;  // padded systems: first true element of each block (device)
   std::map<TripleKey, std::unique_ptr<TripleInfo>> tcache;
+  std::map<const Pattern*, std::unique_ptr<QuadPattern>> qcache;
   // FP64 values (padded blocks)
   double *S = nullptr, *H0 = nullptr, *D[3] = {nullptr, nullptr, nullptr}, *Hm = nullptr;
   double *Sinv = nullptr, *Zs = nullptr, *Xs2 = nullptr;
@@ -170,6 +176,7 @@ struct rt_ctx {
   // the largest pattern and grown outside a capture
   rt::X64Operand xa, xb;
   size_t xa_bytes = 0, xb_bytes = 0;
+  const rt::Pattern* xa_of = nullptr;  // pattern of the operand in xa after a product that split it
   int x_atoms = 0;
   // pinned staging of host copies to and from pageable memory (made by the first large one)
   void* stage = nullptr;
@@ -275,6 +282,13 @@ static Pattern* pattern_for(rt_ctx* c, Sys& s, double r) {
   return raw;
 }
 
+// Quads are taken from this many 4-function triples to a product of quads on:
+// one of 16 x 16 (exact digits on the tensor cores, spgemm13_x64.cu) measured as
+// long as 6.7 real or 5.0 complex 4-function triples on the FP64 pipe (1728 atoms:
+// 0.82 against 0.122 ns, 2.3 against 0.46 ns).  In lattice order there are 9 to 11
+// of them at 8 A, 4.7 at 6 A, 61 in a 64-atom cell.
+constexpr int QUAD_FILL = 6;
+
 static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* B, bool bd, Pattern* C, bool up) {
   TripleKey key{A, B, C, ad, bd, up};
   auto it = s.tcache.find(key);
@@ -306,6 +320,21 @@ static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* 
     int64_t n = 0;
     for (int32_t q : items) n += (int64_t)s.bsize[rowof[q]] * s.bsize[C->h_col[q]];
     ti->true_elems_c = n;
+  }
+  if (s.B == 4 && c->p.precision == RT_FP64) {
+    auto quad = [&](Pattern* P) {
+      std::unique_ptr<QuadPattern>& Q = s.qcache[P];
+      if (!Q) {
+        Q = std::make_unique<QuadPattern>();
+        build_quads(*Q, *P, c->arena, c->ws);
+      }
+      return Q.get();
+    };
+    ti->qa = quad(A);
+    ti->qb = quad(B);
+    ti->qc = quad(C);
+    build_triples(ti->qt, ti->qa->P, ad, ti->qb->P, bd, ti->qc->P, up, c->arena, c->ws);
+    ti->quads = ti->t.n_triples >= (int64_t)QUAD_FILL * ti->qt.n_triples;
   }
   if (ti->t.n_items > s.red_items_n) {
     s.red_items = c->arena.get_n<double>(ti->t.n_items);
@@ -381,9 +410,9 @@ static GemmArgs prepared(rt_ctx* c, Sys& s, TripleInfo& ti, bool fp32, bool cplx
 }
 
 // Room for the split operands of a product over patterns of at most nnzb blocks.
-static void reserve_split(rt_ctx* c, const Sys& s, int64_t nnzb_a, int64_t nnzb_b, bool cplx) {
+static void reserve_split(rt_ctx* c, int n_atoms, int64_t nnzb_a, int64_t nnzb_b, bool cplx) {
   const size_t na = (size_t)nnzb_a * x64_block_bytes(cplx), nb = (size_t)nnzb_b * x64_block_bytes(cplx);
-  if (na <= c->xa_bytes && nb <= c->xb_bytes && s.n_atoms <= c->x_atoms) return;
+  if (na <= c->xa_bytes && nb <= c->xb_bytes && n_atoms <= c->x_atoms) return;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   RT_CUDA_CHECK(cudaStreamIsCapturing(c->ws, &cs));
   RT_REQUIRE(cs == cudaStreamCaptureStatusNone, RT_EINTERNAL, "split operands must be sized before a capture");
@@ -403,30 +432,47 @@ static void reserve_split(rt_ctx* c, const Sys& s, int64_t nnzb_a, int64_t nnzb_
   grow(c->xa.dig, c->xa_bytes, na);
   grow(c->xb.dig, c->xb_bytes, nb);
   size_t ea = (size_t)c->x_atoms * 64, eb = ea;
-  const size_t ne = (size_t)std::max(s.n_atoms, c->x_atoms) * 64;
+  const size_t ne = (size_t)std::max(n_atoms, c->x_atoms) * 64;
   grow(c->xa.exps, ea, ne);
   grow(c->xb.exps, eb, ne);
-  c->x_atoms = std::max(s.n_atoms, c->x_atoms);
+  c->x_atoms = std::max(n_atoms, c->x_atoms);
   c->graph_dirty = true;  // a captured step holds the old addresses
 }
 
-// keep_a: A is the operand of the product just before, unchanged since, so that its split stands
+// keep_a: A is the operand of the product just before, unchanged since, so that its split
+// stands (if that product took the same route, which xa_of says)
 static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cplx, bool ad, bool bd, Epilogue epi,
                  GemmArgs g, const Pattern* C, bool keep_a = false) {
   g = prepared(c, s, ti, fp32, cplx, epi, g, C);
   int B = s.B;
-  if (B == 13 && c->p.precision == RT_FP64) {
-    // 13-function products of the FP64 mode: exact digit products on the tensor cores (6x the CUDA
-    // cores at every size measured, 64 to 512 atoms); the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
-    if (!c->counting) reserve_split(c, s, ti.nnzb_a, ti.nnzb_b, cplx);
+  const Pattern* had = c->xa_of;
+  c->xa_of = nullptr;
+  if ((B == 13 && c->p.precision == RT_FP64) || ti.quads) {
+    // products of the FP64 mode: exact digit products on the tensor cores, of 13-function blocks (6x
+    // the CUDA cores at every size measured, 64 to 512 atoms) and of quads of 4-function blocks;
+    // the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
+    const Pattern &pa = ti.quads ? ti.qa->P : *ti.pa, &pb = ti.quads ? ti.qb->P : *ti.pb;
+    const int32_t *ma = ti.quads ? ti.qa->map : nullptr, *mb = ti.quads ? ti.qb->map : nullptr,
+                  *mc = ti.quads ? ti.qc->map : nullptr;
+    if (ti.quads) {
+      g.item_blk = ti.qt.item_blk;
+      g.ptr = ti.qt.ptr;
+      g.ab = ti.qt.ab;
+      g.n_items = ti.qt.n_items;
+      g.rowidx = ti.qc->P.rowidx;
+      g.colidx = ti.qc->P.col;
+    }
+    if (!c->counting) reserve_split(c, pa.n_atoms, pa.nnzb, pb.nnzb, cplx);
+    keep_a = keep_a && had == &pa;
+    c->xa_of = &pa;
     run(
         c, cls, gemm_flops(ti, cplx), gemm_bytes(s, ti, cplx, fp32),
         [&] {
-          if (!keep_a) launch_split13(g.A, cplx, ad, false, *ti.pa, c->xa, c->ws);
-          launch_split13(g.B, cplx, !bd, true, *ti.pb, c->xb, c->ws);
-          launch_gemm13_x64(cplx, ad, bd, epi, g, c->xa, c->xb, c->ws);
+          const X64Split ops[2] = {{g.B, &pb, mb, !bd, true, c->xb}, {g.A, &pa, ma, ad, false, c->xa}};
+          launch_split13(ops, keep_a ? 1 : 2, cplx, c->ws);
+          launch_gemm13_x64(cplx, ad, bd, epi, g, c->xa, c->xb, mc, c->ws);
         },
-        keep_a ? 2 : 3);
+        2);
     return;
   }
   RT_REQUIRE(!g.a_planar || (fp32 && cplx && B == 13 && !ti.tiles.built), RT_EINTERNAL,
@@ -481,7 +527,7 @@ static GemmArgs args(const void* A, const void* B, void* C) {
 static void residual_from_items(rt_ctx* c, Sys& s, const TripleInfo& ti, double* out, double* out2) {
   run(
       c, PC_MISC, 0, 0,
-      [&] { launch_sum(s.red_items, ti.t.n_items, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
+      [&] { launch_sum(s.red_items, ti.quads ? ti.qt.n_items : ti.t.n_items, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
 }
 
 // ----------------------------------------------------------------------------
@@ -737,7 +783,14 @@ static void setup_system(rt_ctx* c, Sys& s, const rt_system& in) {
     // the captured step holds FP64 products: their split operands are sized here
     int64_t most = 0;
     for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
-    reserve_split(c, s, most, most, true);
+    reserve_split(c, s.n_atoms, most, most, true);
+  }
+  if (s.B == 4 && p.precision == RT_FP64) {
+    int64_t most = 0;
+    for (const auto& q : s.qcache) most = std::max(most, q.second->P.nnzb);
+    bool any = false;
+    for (const auto& ti : s.tcache) any = any || ti.second->quads;
+    if (any) reserve_split(c, (s.n_atoms + 3) / 4, most, most, true);
   }
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
@@ -2633,9 +2686,21 @@ rt_status rt_debug_check(rt_ctx* c, int64_t* n_checked) {
     int64_t n = 0;
     for (size_t si = 0; si < c->sys.size(); ++si) {
       Sys& s = *c->sys[si];
+      struct List {
+        TripleKey key;
+        const Triples* t;
+        int n_atoms;
+      };
+      std::vector<List> lists;
       for (auto& kv : s.tcache) {
-        const TripleKey& key = kv.first;
-        const Triples& T = kv.second->t;
+        const TripleKey& k = kv.first;
+        const TripleInfo& ti = *kv.second;
+        lists.push_back({k, &ti.t, s.n_atoms});
+        if (ti.qa) lists.push_back({{&ti.qa->P, &ti.qb->P, &ti.qc->P, k.ad, k.bd, k.up}, &ti.qt, (s.n_atoms + 3) / 4});
+      }
+      for (const List& list : lists) {
+        const TripleKey& key = list.key;
+        const Triples& T = *list.t;
         std::vector<int32_t> items((size_t)T.n_items);
         std::vector<int64_t> ptr((size_t)T.n_items + 1, 0);
         std::vector<int32_t> ab((size_t)(2 * T.n_triples));
@@ -2651,7 +2716,7 @@ rt_status rt_debug_check(rt_ctx* c, int64_t* n_checked) {
         int64_t bad = -1;
         std::string why;
         const bool ok = check_triples_host(
-            s.n_atoms, key.A->h_rowptr.data(), key.A->h_col.data(), key.ad, key.B->h_rowptr.data(),
+            list.n_atoms, key.A->h_rowptr.data(), key.A->h_col.data(), key.ad, key.B->h_rowptr.data(),
             key.B->h_col.data(), key.bd, key.C->h_rowptr.data(), key.C->h_col.data(), key.up, T.n_items, items.data(),
             ptr.data(), ab.data(), T.n_triples, &bad, &why);
         RT_REQUIRE(ok, RT_EINTERNAL,

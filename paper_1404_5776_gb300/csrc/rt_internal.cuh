@@ -224,13 +224,28 @@ struct X64Operand {
   int32_t* exps = nullptr;       // [n_atoms][16] biased exponent of each scale
 };
 size_t x64_block_bytes(bool cplx);
-// The scaled index is the row of the stored blocks, or (by_col) their column:
-// op(A) takes rows as stored and columns daggered, op(B) the other way round.
-// right: the operand order of op(B).
-void launch_split13(const void* vals, bool cplx, bool by_col, bool right, const Pattern& P, const X64Operand& out,
-                    cudaStream_t st);
+// One operand to split.  The scaled index is the row of the stored blocks, or
+// (by_col) their column: op(A) takes rows as stored and columns daggered, op(B)
+// the other way round.  right: the operand order of op(B).  quad_map: 4-function
+// blocks taken as quads, P then being their pattern (below).
+struct X64Split {
+  const void* vals;
+  const Pattern* P;
+  const int32_t* quad_map;
+  bool by_col, right;
+  X64Operand out;
+};
+void launch_split13(const X64Split* ops, int n, bool cplx, cudaStream_t st);  // one or two operands of one system
 void launch_gemm13_x64(bool cplx, bool a_dag, bool b_dag, Epilogue epi, const GemmArgs& g, const X64Operand& A,
-                       const X64Operand& B, cudaStream_t st);
+                       const X64Operand& B, const int32_t* quad_cmap, cudaStream_t st);
+
+// Quads of a 4-function pattern: groups of four consecutive atoms as atoms of 16
+// functions; a quad exists where any of its 16 blocks does, and map names them.
+struct QuadPattern {
+  Pattern P;               // over (n_atoms + 3) / 4 groups
+  int32_t* map = nullptr;  // [P.nnzb][4 row atoms][4 column atoms] block of the pattern, -1: none
+};
+void build_quads(QuadPattern& Q, const Pattern& P, Arena& arena, cudaStream_t st);
 
 // Launches; `cplx` selects complex values, `b_dag` conj-transposes B's blocks,
 // `a_dag` A's blocks.  Element type by precision: FP64 double/double2, FP32 float/float2.

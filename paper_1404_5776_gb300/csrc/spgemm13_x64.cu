@@ -1,4 +1,5 @@
-// FP64 block products of 13-function atoms on the tensor cores.
+// FP64 block products on the tensor cores: 13-function atoms, and 4-function atoms
+// in quads.
 //
 // Same contraction as spgemm.cu (C_ij = sum_k op(A)_ik op(B)_kj over the triple
 // list of the output block).  GB300 does two FP64 fused multiply-adds per clock
@@ -42,7 +43,14 @@
 // times slower.  What bounds it: the tensor pipe (52-70 % busy in the Taylor
 // powers), with the wait for the next blocks' first digits beside it.
 // 216 atoms x 13, r = 8 A: a Taylor power 8.9 -> 1.14 ms with its splits, M = U K
-// 21.7 -> 3.3 ms; FP64 EM step at 512 atoms 126 -> 20.5 ms.
+// 21.7 -> 3.3 ms; FP64 EM step at 512 atoms 126 -> 20.5 ms.  The time follows the
+// warps in flight: A's digits in two sets of registers (12 warps) took 27 % longer,
+// five CTAs of 96 registers (spills) 65 %.
+//
+// 4-function atoms take the same kernel in quads: the blocks between two groups of
+// four consecutive atoms as one 16 x 16 block, absent ones zero (a 4 x 4 triple
+// alone would fill an eighth of a product).  FP64 EM step of 1728 atoms x 4 at 8 A:
+// 12.4 -> 7.0 ms; of 64 atoms x 4: 0.41 -> 0.18 ms.
 #include <algorithm>
 
 #include "rt_internal.cuh"
@@ -51,13 +59,24 @@ namespace rt {
 
 namespace x64 {
 
-constexpr int BS = 13;
-constexpr int NE = BS * BS;
+// A block of the product: a 13-function block as stored, or a quad: the 4-function
+// blocks between two groups of four consecutive atoms as one 16 x 16 block (absent
+// ones are zero).
+template <bool QUAD>
+struct Shape {
+  static constexpr int BS = QUAD ? 16 : 13;
+  static constexpr int NE = BS * BS;
+};
 constexpr int BLK = 4096;      // bytes of one split real block: 8 digits x 32 lanes x 8 elements in FP16
 constexpr int WARPS = 4;
 constexpr int MINB = 4;
+// warps of a CTA: an item takes 2 (real) or 4 (complex) for each share of its triples
+template <bool CPLX, int KS>
+constexpr int CTA_WARPS = (CPLX ? 4 : 2) * KS > WARPS ? (CPLX ? 4 : 2) * KS : WARPS;
 constexpr int NW = 9;          // weights p + q of the digit pairs that are multiplied
-constexpr int CARRY = 8;       // real products between two carries: 13 * 8 * 2^14 * 8 + carries < 2^24
+// real products between two carries: (13 or 16) * 8 * 2^14 * CARRY + the carries < 2^24
+template <bool QUAD>
+constexpr int CARRY = QUAD ? 6 : 8;
 constexpr int EXP_NAN = 2047;  // scale of a row that holds a NaN or an infinity: its products are NaN
 constexpr int MAX_LEAD = 9;    // a block with so many leading zero digits adds nothing (NW weights)
 constexpr int SPLIT_WARPS = 16;
@@ -89,36 +108,68 @@ __device__ __forceinline__ unsigned less_1152(unsigned h) {
   return r;
 }
 
-template <bool CPLX>
-__global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const double* __restrict__ vals,
-                                                              const int32_t* __restrict__ rowptr,
-                                                              const int32_t* __restrict__ tmap, int by_col, int right,
-                                                              unsigned char* __restrict__ dig,
-                                                              unsigned char* __restrict__ lead,
-                                                              int32_t* __restrict__ exps) {
+// Element (x, y) of block q: in the stored blocks, or (quads) in the 4-function
+// block that the map names for its two atoms (-1: none, zero).
+template <bool QUAD>
+__device__ __forceinline__ int64_t element(const int32_t* __restrict__ map, int64_t q, int x, int y) {
+  if constexpr (QUAD) {
+    const int blk = map[q * 16 + (x >> 2) * 4 + (y >> 2)];
+    return blk < 0 ? -1 : (int64_t)blk * 16 + (x & 3) * 4 + (y & 3);
+  } else {
+    return q * 169 + x * 13 + y;
+  }
+}
+
+struct SplitArgs {  // one operand; a launch takes one or two (blockIdx.y)
+  const double* vals;
+  const int32_t* map;
+  const int32_t* rowptr;
+  const int32_t* tmap;
+  int by_col, right;
+  unsigned char* dig;
+  unsigned char* lead;
+  int32_t* exps;
+};
+struct SplitPair {
+  SplitArgs s[2];
+};
+
+template <bool CPLX, bool QUAD>
+__global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const __grid_constant__ SplitPair pair) {
+  const SplitArgs& s = pair.s[blockIdx.y];
+  const double* __restrict__ vals = s.vals;
+  const int32_t* __restrict__ map = s.map;
+  const int32_t* __restrict__ rowptr = s.rowptr;
+  const int32_t* __restrict__ tmap = s.tmap;
+  const int by_col = s.by_col, right = s.right;
+  unsigned char* __restrict__ dig = s.dig;
+  unsigned char* __restrict__ lead = s.lead;
+  int32_t* __restrict__ exps = s.exps;
   constexpr int NC = CPLX ? 2 : 1;
+  constexpr int BS = Shape<QUAD>::BS, NE = Shape<QUAD>::NE;
   __shared__ int smax[16];
   const int atom = blockIdx.x;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int q0 = rowptr[atom], q1 = rowptr[atom + 1];
   if (threadIdx.x < 16) smax[threadIdx.x] = 1;
   __syncthreads();
-  constexpr int EPT = (NE + 31) / 32;
+  constexpr int EPT = (NE + 31) / 32;  // 13: elements e = lane + 32 k keep their row and column from block to block
   int mx[EPT];
 #pragma unroll
   for (int k = 0; k < EPT; ++k) mx[k] = 1;
   for (int q = q0 + warp; q < q1; q += SPLIT_WARPS) {
-    const double* v = vals + (int64_t)(by_col ? tmap[q] : q) * NE * NC;
+    const int qb = by_col ? tmap[q] : q;
 #pragma unroll
     for (int k = 0; k < EPT; ++k) {
       const int e = lane + 32 * k;
-      if (e < NE) {
+      const int64_t at = e < NE ? element<QUAD>(map, qb, e / BS, e % BS) : -1;
+      if (at >= 0) {
         int m;
         if constexpr (CPLX) {
-          const double2 z = reinterpret_cast<const double2*>(v)[e];
+          const double2 z = reinterpret_cast<const double2*>(vals)[at];
           m = max(__double2hiint(z.x) & 0x7fffffff, __double2hiint(z.y) & 0x7fffffff);
         } else {
-          m = __double2hiint(v[e]) & 0x7fffffff;
+          m = __double2hiint(vals[at]) & 0x7fffffff;
         }
         mx[k] = max(mx[k], m >> 20);
       }
@@ -135,20 +186,19 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const double* __re
   const int g = lane >> 2, t = lane & 3;
   for (int q = q0 + warp; q < q1; q += SPLIT_WARPS) {
     const int qb = by_col ? tmap[q] : q;
-    const double* v = vals + (int64_t)qb * NE * NC;
     double val[NC][8];
 #pragma unroll
     for (int f = 0; f < 8; ++f) {
       const int m = g + ((f >> 1) & 1) * 8;               // scaled index
       const int k = 2 * t + (f & 1) + (f >> 2) * 8;       // summed index
       const bool in = m < BS && k < BS && smax[m] != EXP_NAN;
-      const int e = by_col ? k * BS + m : m * BS + k;
+      const int64_t at = in ? element<QUAD>(map, qb, by_col ? k : m, by_col ? m : k) : -1;
       if constexpr (CPLX) {
-        const double2 z = in ? reinterpret_cast<const double2*>(v)[e] : make_double2(0.0, 0.0);
+        const double2 z = at >= 0 ? reinterpret_cast<const double2*>(vals)[at] : make_double2(0.0, 0.0);
         val[0][f] = z.x;
         val[1][f] = z.y;
       } else {
-        val[0][f] = in ? v[e] : 0.0;
+        val[0][f] = at >= 0 ? vals[at] : 0.0;
       }
     }
 #pragma unroll
@@ -209,6 +259,7 @@ struct Args {
   const unsigned char* lB;
   const int32_t* eA;
   const int32_t* eB;
+  const int32_t* cmap;  // quads: the output's 4-function blocks
 };
 
 __device__ __forceinline__ void mma16816(float (&c)[4], const uint4& a, unsigned b0, unsigned b1) {
@@ -232,45 +283,52 @@ __device__ __forceinline__ int small_int(float v) { return __float_as_int(v + 12
 // at zero.  A digit's registers take the next product's digit (na, nb; weights
 // from znext on) right after their last use here, so that the loads are in
 // flight under the multiplications that follow.
-template <int Z>
+// ALL: every digit is loaded, also those below the last weight (a real product's
+// warp is bound by its instructions: 3 % faster; a complex one's by its loads:
+// 7 % slower).
+template <int Z, bool ALL>
 __device__ __forceinline__ void multiply(float (&acc)[NW][4], uint4 (&a)[8], uint4 (&b)[4],
                                          const uint4* __restrict__ na, const uint4* __restrict__ nb, int znext) {
   constexpr int LAST = NW - 1 - Z;  // p + q <= LAST
 #pragma unroll
   for (int p = 7; p >= 0; --p)
-    if (p > LAST && p + znext < NW) a[p] = na[32 * p];
+    if (p > LAST && (ALL || p + znext < NW)) a[p] = na[32 * p];
 #pragma unroll
   for (int q2 = 3; q2 >= 0; --q2)
-    if (2 * q2 > LAST && 2 * q2 + znext < NW) b[q2] = nb[32 * q2];
+    if (2 * q2 > LAST && (ALL || 2 * q2 + znext < NW)) b[q2] = nb[32 * q2];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     if (q <= LAST) {
       const unsigned b0 = (q & 1) ? b[q >> 1].z : b[q >> 1].x, b1 = (q & 1) ? b[q >> 1].w : b[q >> 1].y;
 #pragma unroll
-      for (int p = 0; p < 8; ++p)
+      for (int p = 7; p >= 0; --p)  // the digits of A that the last product left first come first
         if (p + q <= LAST) mma16816(acc[p + q + Z], a[p], b0, b1);
-      if (((q & 1) || q == LAST) && (q & ~1) + znext < NW) b[q >> 1] = nb[32 * (q >> 1)];
+      if (((q & 1) || q == LAST) && (ALL || (q & ~1) + znext < NW)) b[q >> 1] = nb[32 * (q >> 1)];
 #pragma unroll
       for (int p = 7; p >= 0; --p)
-        if (p <= LAST && (LAST - p < 7 ? LAST - p : 7) == q && p + znext < NW) a[p] = na[32 * p];
+        if (p <= LAST && (LAST - p < 7 ? LAST - p : 7) == q && (ALL || p + znext < NW)) a[p] = na[32 * p];
     }
   }
 }
 
-template <bool CPLX, bool ADAG, bool BDAG, int EPI>
-__global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_constant__ Args x) {
+template <bool CPLX, bool ADAG, bool BDAG, int EPI, bool QUAD, int KS>
+__global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_WARPS<CPLX, KS>) k_gemm13_x64(const __grid_constant__ Args x) {
   constexpr int NP = CPLX ? 2 : 1;  // real products per triple and warp; parts of a complex output
-  constexpr int WPI = 2 * NP;       // warps per item: 8-column halves x parts
+  constexpr int WPB = 2 * NP;       // warps of one share of an item: 8-column halves x parts
+  constexpr int WPI = WPB * KS;     // warps per item
+  constexpr int NWARP = CTA_WARPS<CPLX, KS>;
+  constexpr int BS = Shape<QUAD>::BS, NE = Shape<QUAD>::NE;
   const GemmArgs& g = x.g;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const int half = warp & 1;                      // output columns 8 half .. 8 half + 7
   const int part = CPLX ? ((warp >> 1) & 1) : 0;  // 0: real part, 1: imaginary part
-  const int slot = warp / WPI;
-  const int64_t item = (int64_t)blockIdx.x * (WARPS / WPI) + slot;
+  const int slot = warp / WPI, ks = KS > 1 ? (warp % WPI) / WPB : 0;
+  const int64_t item = (int64_t)blockIdx.x * (NWARP / WPI) + slot;
   if (item >= g.n_items) return;  // the warps of one item leave together
 
-  __shared__ double sC[WARPS / WPI][NE * NP];
+  __shared__ double sC[NWARP / WPI][NE * NP];
+  __shared__ long long shares[KS > 1 ? (KS - 1) * WPB : 1][KS > 1 ? 8 : 1][32];  // integer sums of the shares after the first (one item a CTA)
 
   // signs of the two real products of this part (op(A) = Ar + i sa Ai, op(B) = Br + i sb Bi):
   //   real part:       Ar Br - sa sb Ai Bi;   imaginary part: sb Ar Bi + sa Ai Br
@@ -298,8 +356,14 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
       }
   };
 
-  const int64_t t0 = g.ptr[item], t1 = g.ptr[item + 1];
-  const int2* __restrict__ ab = g.ab;
+  const int64_t t0 = g.ptr[item];
+  int nt = (int)(g.ptr[item + 1] - t0);
+  const int2* __restrict__ ab = g.ab + t0;
+  if constexpr (KS > 1) {  // this warp's share of the triples
+    const int share = (nt + KS - 1) / KS, first = min(nt, share * ks);
+    ab += first;
+    nt = min(share, nt - first);
+  }
   const unsigned char* __restrict__ dA = x.dA + lane * 16;
   const unsigned char* __restrict__ dB = x.dB + lane * 16 + half * (BLK / 2);
   // digits to skip of a triple's blocks: bytes 0, 1: A's parts, bytes 2, 3: B's
@@ -312,9 +376,9 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
   };
   auto lead_a = [&](unsigned z, int sub) { return (int)((z >> (8 * sub)) & 0xff); };
   auto lead_b = [&](unsigned z, int sub) { return (int)((z >> (16 + 8 * (CPLX ? (sub ^ part) : 0))) & 0xff); };
-  if (t0 < t1) {
+  if (nt > 0) {
     // triples t, t + 1 and t + 2 of the list; the digits to skip of the first two
-    int2 cur = ab[t0], nxt = t0 + 1 < t1 ? ab[t0 + 1] : cur, nxt2 = t0 + 2 < t1 ? ab[t0 + 2] : nxt;
+    int2 cur = ab[0], nxt = 1 < nt ? ab[1] : cur, nxt2 = 2 < nt ? ab[2] : nxt;
     unsigned zc = leads(cur), zn = leads(nxt);
     uint4 a[8], b[4];
     {
@@ -326,8 +390,8 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
       for (int p = 0; p < 4; ++p) b[p] = pb[32 * p];
     }
     int since = 0;
-    for (int64_t t = t0; t < t1; ++t) {
-      const int2 nxt3 = t + 3 < t1 ? ab[t + 3] : nxt2;
+    for (int t = 0; t < nt; ++t) {
+      const int2 nxt3 = t + 3 < nt ? ab[t + 3] : nxt2;
       const unsigned zn2 = leads(nxt2);
 #pragma unroll
       for (int sub = 0; sub < NP; ++sub) {
@@ -349,19 +413,23 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
             a[p].w ^= 0x80008000u;
           }
         }
+        // the digits of A that this product needs longest are loaded last and needed first: into L1
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+          if (p + znext < NW) asm volatile("prefetch.global.L1 [%0];" ::"l"(na + 32 * p));
         switch (zz) {
-          case 0: multiply<0>(acc, a, b, na, nbp, znext); break;
-          case 1: multiply<1>(acc, a, b, na, nbp, znext); break;
-          case 2: multiply<2>(acc, a, b, na, nbp, znext); break;
-          case 3: multiply<3>(acc, a, b, na, nbp, znext); break;
-          case 4: multiply<4>(acc, a, b, na, nbp, znext); break;
-          case 5: multiply<5>(acc, a, b, na, nbp, znext); break;
-          case 6: multiply<6>(acc, a, b, na, nbp, znext); break;
-          case 7: multiply<7>(acc, a, b, na, nbp, znext); break;
-          case 8: multiply<8>(acc, a, b, na, nbp, znext); break;
-          default: multiply<NW>(acc, a, b, na, nbp, znext); break;  // below every weight: nothing but the loads
+          case 0: multiply<0, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 1: multiply<1, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 2: multiply<2, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 3: multiply<3, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 4: multiply<4, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 5: multiply<5, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 6: multiply<6, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 7: multiply<7, !CPLX>(acc, a, b, na, nbp, znext); break;
+          case 8: multiply<8, !CPLX>(acc, a, b, na, nbp, znext); break;
+          default: multiply<NW, !CPLX>(acc, a, b, na, nbp, znext); break;  // below every weight: nothing but the loads
         }
-        if (++since == CARRY) {
+        if (++since == CARRY<QUAD>) {
           carry();
           since = 0;
         }
@@ -377,22 +445,45 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
 
   const int q = g.item_blk[item];
   const int i = g.rowidx[q], j = g.colidx[q];
-  {
+  // the weights as two integers, hi 2^48 + lo in units of 256^6 2^-124
+  long long hi[4], lo[4];
+#pragma unroll
+  for (int rr = 0; rr < 4; ++rr) {
+    const int lo1 = (small_int(acc[3][rr]) * 256 + small_int(acc[4][rr])) * 256 + small_int(acc[5][rr]);
+    const int lo0 = (small_int(acc[6][rr]) * 256 + small_int(acc[7][rr])) * 256 + small_int(acc[8][rr]);
+    const int hi1 = __float2int_rn(top[rr]);
+    const int hi0 = (small_int(acc[0][rr]) * 256 + small_int(acc[1][rr])) * 256 + small_int(acc[2][rr]);
+    lo[rr] = (long long)lo1 * (1 << 24) + lo0;
+    hi[rr] = (long long)hi1 * (1 << 24) + hi0;
+  }
+  if constexpr (KS > 1) {
+    const int base = warp % WPB;
+    if (ks > 0)
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) {
+        shares[(ks - 1) * WPB + base][rr][lane] = hi[rr];
+        shares[(ks - 1) * WPB + base][4 + rr][lane] = lo[rr];
+      }
+    asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPI) : "memory");
+    if (ks == 0)
+#pragma unroll
+      for (int k = 1; k < KS; ++k)
+#pragma unroll
+        for (int rr = 0; rr < 4; ++rr) {
+          hi[rr] += shares[(k - 1) * WPB + base][rr][lane];
+          lo[rr] += shares[(k - 1) * WPB + base][4 + rr][lane];
+        }
+  }
+  if (ks == 0) {
     const int gr = lane >> 2, tc = lane & 3;
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr) {
       const int r = gr + (rr >> 1) * 8, c = 8 * half + 2 * tc + (rr & 1);
       if (r < BS && c < BS) {
-        // (hi 2^48 + lo) 256^6 2^-124: the integers enter FP64 as mantissas of 1.5 2^24 and
-        // 1.5 2^-24 (exact), and meet with one rounding
-        const int lo1 = (small_int(acc[3][rr]) * 256 + small_int(acc[4][rr])) * 256 + small_int(acc[5][rr]);
-        const int lo0 = (small_int(acc[6][rr]) * 256 + small_int(acc[7][rr])) * 256 + small_int(acc[8][rr]);
-        const int hi1 = __float2int_rn(top[rr]);
-        const int hi0 = (small_int(acc[0][rr]) * 256 + small_int(acc[1][rr])) * 256 + small_int(acc[2][rr]);
-        const long long lo = (long long)lo1 * (1 << 24) + lo0, hi = (long long)hi1 * (1 << 24) + hi0;
+        // the integers enter FP64 as mantissas of 1.5 2^24 and 1.5 2^-24 (exact), and meet with one rounding
         constexpr double MH = 0x1.8p24, ML = 0x1.8p-24;
-        const double vh = __longlong_as_double(__double_as_longlong(MH) + hi) - MH;
-        const double vl = __longlong_as_double(__double_as_longlong(ML) + lo) - ML;
+        const double vh = __longlong_as_double(__double_as_longlong(MH) + hi[rr]) - MH;
+        const double vl = __longlong_as_double(__double_as_longlong(ML) + lo[rr]) - ML;
         sC[slot][(r * BS + c) * NP + part] = pow2_scaled(vh + vl, x.eA[i * 16 + r], x.eB[j * 16 + c]);
       }
     }
@@ -404,35 +495,36 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
   const int el = lane + 32 * (warp % WPI);  // this thread's first element
   constexpr int STEP = 32 * WPI;
   V* __restrict__ C = static_cast<V*>(g.C);
-  if constexpr (EPI == EPI_STORE) {
-    for (int e = el; e < NE; e += STEP) C[(int64_t)q * NE + e] = val[e];
-  } else if constexpr (EPI == EPI_ADD) {
+  if constexpr (EPI == EPI_STORE || EPI == EPI_ADD || EPI == EPI_STORE_ACC) {
     for (int e = el; e < NE; e += STEP) {
-      if constexpr (CPLX) {
-        const double2 o = C[(int64_t)q * NE + e];
-        C[(int64_t)q * NE + e] = make_double2(o.x + val[e].x, o.y + val[e].y);
+      const int r = e / BS, c = e - r * BS;
+      const int64_t at = element<QUAD>(x.cmap, q, r, c);
+      if (QUAD && at < 0) continue;
+      if constexpr (EPI == EPI_STORE) {
+        C[at] = val[e];
+      } else if constexpr (EPI == EPI_ADD) {
+        if constexpr (CPLX) {
+          const double2 o = C[at];
+          C[at] = make_double2(o.x + val[e].x, o.y + val[e].y);
+        } else {
+          C[at] += val[e];
+        }
       } else {
-        C[(int64_t)q * NE + e] += val[e];
-      }
-    }
-  } else if constexpr (EPI == EPI_STORE_ACC) {
-    // real power T^n stored (unless C is null); coef * T^n added to complex U
-    double2* __restrict__ U = static_cast<double2*>(g.U);
-    const int uq = g.umap ? g.umap[q] : q;
-    for (int e = el; e < NE; e += STEP) {
-      if (C) C[(int64_t)q * NE + e] = val[e];
-      if (uq >= 0) {
-        double2 u = U[(int64_t)uq * NE + e];
+        // real power T^n stored (unless C is null); coef * T^n added to complex U (on the same pattern)
+        if (C) C[at] = val[e];
+        double2* __restrict__ U = static_cast<double2*>(g.U);
+        double2 u = U[at];
         if (g.coef_imag) u.y += g.coef * val[e];
         else u.x += g.coef * val[e];
-        U[(int64_t)uq * NE + e] = u;
+        U[at] = u;
       }
     }
   } else if constexpr (EPI == EPI_TWO_I) {
-    const int bi = g.bsize[i], bj = g.bsize[j];
     double part_sum = 0.0;
     for (int e = el; e < NE; e += STEP) {
       const int r = e / BS, c = e - r * BS;
+      const int64_t at = element<QUAD>(x.cmap, q, r, c);
+      if (QUAD && at < 0) continue;
       double re, im = 0.0;
       if constexpr (CPLX) {
         re = val[e].x;
@@ -442,12 +534,13 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
       }
       const bool on = i == j && r == c;
       const double dre = (on ? 1.0 : 0.0) - re;
-      if (r < bi && c < bj) part_sum += dre * dre + im * im;
-      if constexpr (CPLX) C[(int64_t)q * NE + e] = make_double2((on ? 2.0 : 0.0) - re, -im);
-      else C[(int64_t)q * NE + e] = (on ? 2.0 : 0.0) - re;
+      const int bi = QUAD ? g.bsize[4 * i + (r >> 2)] : g.bsize[i], bj = QUAD ? g.bsize[4 * j + (c >> 2)] : g.bsize[j];
+      if ((QUAD ? (r & 3) : r) < bi && (QUAD ? (c & 3) : c) < bj) part_sum += dre * dre + im * im;
+      if constexpr (CPLX) C[at] = make_double2((on ? 2.0 : 0.0) - re, -im);
+      else C[at] = (on ? 2.0 : 0.0) - re;
     }
     for (int off = 16; off > 0; off >>= 1) part_sum += __shfl_down_sync(0xffffffffu, part_sum, off);
-    __shared__ double partial[WARPS];
+    __shared__ double partial[NWARP];
     if (lane == 0) partial[warp] = part_sum;
     asm volatile("bar.sync %0, %1;" ::"r"(slot + 1), "n"(32 * WPI) : "memory");
     if (lane == 0 && warp % WPI == 0) {
@@ -456,24 +549,38 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
       g.red[item] = sum;
     }
   } else if constexpr (EPI == EPI_SANDWICH) {
-    // K'_ij for j >= i; mirror K'_ji = K'_ij^dagger; hermitian diagonal blocks
+    // K'_ij for j >= i; mirror K'_ji = K'_ij^dagger; hermitian diagonal blocks (atoms i, j: a
+    // quad of two different groups lies above the diagonal as a whole)
     if (i != j) {
-      const int qt = g.tmap[q];
       for (int e = el; e < NE; e += STEP) {
         const int r = e / BS, c = e - r * BS;
-        C[(int64_t)q * NE + e] = val[e];
-        // the mirror, written in its own order: element (r,c) of block (j,i)
-        const double2 m = val[c * BS + r];
-        C[(int64_t)qt * NE + e] = make_double2(m.x, -m.y);
+        const int64_t at = element<QUAD>(x.cmap, q, r, c);
+        if (QUAD && at < 0) continue;
+        C[at] = val[e];
+        if constexpr (QUAD) {
+          C[(int64_t)g.tmap[at >> 4] * 16 + (c & 3) * 4 + (r & 3)] = make_double2(val[e].x, -val[e].y);
+        } else {
+          // the mirror, written in its own order: element (r,c) of block (j,i)
+          const double2 m = val[c * BS + r];
+          C[(int64_t)g.tmap[q] * NE + e] = make_double2(m.x, -m.y);
+        }
       }
     } else {
       double herm = 0.0;
       for (int e = el; e < NE; e += STEP) {
         const int r = e / BS, c = e - r * BS;
-        const double2 v = val[e], tv = val[c * BS + r];
+        const int64_t at = element<QUAD>(x.cmap, q, r, c);
+        if (QUAD && (at < 0 || (r >> 2) > (c >> 2))) continue;
+        const double2 v = val[e];
+        if (QUAD && (r >> 2) < (c >> 2)) {
+          C[at] = v;
+          C[(int64_t)g.tmap[at >> 4] * 16 + (c & 3) * 4 + (r & 3)] = make_double2(v.x, -v.y);
+          continue;
+        }
+        const double2 tv = val[c * BS + r];
         const double dr = v.x - tv.x, di = v.y + tv.y;  // K - K^dagger
         herm = fmax(herm, sqrt(dr * dr + di * di));
-        C[(int64_t)q * NE + e] = make_double2(0.5 * (v.x + tv.x), 0.5 * (v.y - tv.y));
+        C[at] = make_double2(0.5 * (v.x + tv.x), 0.5 * (v.y - tv.y));
       }
       for (int off = 16; off > 0; off >>= 1) herm = fmax(herm, __shfl_xor_sync(0xffffffffu, herm, off));
       if (lane == 0 && g.herm_max) atomicMax(g.herm_max, (unsigned long long)__double_as_longlong(herm));
@@ -481,36 +588,55 @@ __global__ void __launch_bounds__(WARPS * 32, MINB) k_gemm13_x64(const __grid_co
   }
 }
 
-template <bool CPLX, bool ADAG, bool BDAG, int EPI>
-static void launch(const Args& x, cudaStream_t st) {
-  const int64_t per = WARPS / (CPLX ? 4 : 2);
+template <bool CPLX, bool ADAG, bool BDAG, int EPI, int KS>
+static void launch_ks(const Args& x, cudaStream_t st) {
+  constexpr int W = CTA_WARPS<CPLX, KS>;
+  const int64_t per = W / ((CPLX ? 4 : 2) * KS);
   const int64_t grid = (x.g.n_items + per - 1) / per;
   RT_REQUIRE(grid < (1ll << 31), RT_EINTERNAL, "grid too large");
-  k_gemm13_x64<CPLX, ADAG, BDAG, EPI><<<(unsigned)grid, WARPS * 32, 0, st>>>(x);
+  if (x.cmap) k_gemm13_x64<CPLX, ADAG, BDAG, EPI, true, KS><<<(unsigned)grid, W * 32, 0, st>>>(x);
+  else k_gemm13_x64<CPLX, ADAG, BDAG, EPI, false, KS><<<(unsigned)grid, W * 32, 0, st>>>(x);
   RT_CUDA_CHECK(cudaGetLastError());
+}
+
+// A product whose warps leave most of the chip idle shares each item's triples
+// between KS times the warps (the integer sums of the shares add up exactly, so
+// the result does not depend on KS): as long as all of them are resident at once,
+// 16 warps on each of 152 SMs.
+template <bool CPLX, bool ADAG, bool BDAG, int EPI>
+static void launch(const Args& x, cudaStream_t st) {
+  const int64_t warps = x.g.n_items * (CPLX ? 4 : 2);
+  if (4 * warps <= 152 * 16) return launch_ks<CPLX, ADAG, BDAG, EPI, 4>(x, st);
+  if (2 * warps <= 152 * 16) return launch_ks<CPLX, ADAG, BDAG, EPI, 2>(x, st);
+  launch_ks<CPLX, ADAG, BDAG, EPI, 1>(x, st);
 }
 
 }  // namespace x64
 
 size_t x64_block_bytes(bool cplx) { return (size_t)x64::BLK * (cplx ? 2 : 1); }
 
-void launch_split13(const void* vals, bool cplx, bool by_col, bool right, const Pattern& P, const X64Operand& out,
-                    cudaStream_t st) {
-  if (P.nnzb == 0 || P.n_atoms == 0) return;
-  if (cplx)
-    x64::k_split13<true><<<P.n_atoms, x64::SPLIT_WARPS * 32, 0, st>>>(static_cast<const double*>(vals), P.rowptr, P.tmap,
-                                                                      by_col, right, out.dig, out.lead, out.exps);
-  else
-    x64::k_split13<false><<<P.n_atoms, x64::SPLIT_WARPS * 32, 0, st>>>(static_cast<const double*>(vals), P.rowptr,
-                                                                       P.tmap, by_col, right, out.dig, out.lead, out.exps);
+void launch_split13(const X64Split* ops, int n, bool cplx, cudaStream_t st) {
+  using namespace x64;
+  SplitPair pair{};
+  for (int k = 0; k < n; ++k) {
+    const X64Split& o = ops[k];
+    pair.s[k] = {static_cast<const double*>(o.vals), o.quad_map,   o.P->rowptr, o.P->tmap, o.by_col, o.right,
+                 o.out.dig,                          o.out.lead, o.out.exps};
+  }
+  const int atoms = ops[0].P->n_atoms;  // both operands: the same system
+  if (n == 0 || atoms == 0) return;
+  auto go = [&](auto kernel) { kernel<<<dim3(atoms, n), SPLIT_WARPS * 32, 0, st>>>(pair); };
+  if (ops[0].quad_map) cplx ? go(k_split13<true, true>) : go(k_split13<false, true>);
+  else cplx ? go(k_split13<true, false>) : go(k_split13<false, false>);
   RT_CUDA_CHECK(cudaGetLastError());
 }
 
 void launch_gemm13_x64(bool cplx, bool a_dag, bool b_dag, Epilogue epi, const GemmArgs& g, const X64Operand& A,
-                       const X64Operand& B, cudaStream_t st) {
+                       const X64Operand& B, const int32_t* quad_cmap, cudaStream_t st) {
   using namespace x64;
   if (g.n_items == 0) return;
-  const Args x{g, A.dig, B.dig, A.lead, B.lead, A.exps, B.exps};
+  RT_REQUIRE(epi != EPI_STORE_ACC || (!g.umap && g.U), RT_EINTERNAL, "the Taylor accumulator lies on the output pattern");
+  const Args x{g, A.dig, B.dig, A.lead, B.lead, A.exps, B.exps, quad_cmap};
   if (!cplx && !a_dag && !b_dag) {
     if (epi == EPI_STORE) return launch<false, false, false, EPI_STORE>(x, st);
     if (epi == EPI_STORE_ACC) return launch<false, false, false, EPI_STORE_ACC>(x, st);

@@ -1,4 +1,5 @@
-"""FP64 products of 13-function atoms by exact digit products (tensor cores).
+"""FP64 products by exact digit products (tensor cores): 13-function blocks, and
+4-function blocks in quads of four consecutive atoms.
 
 The digits are exact, so a product with the identity has to return the other
 operand bit for bit wherever its entries keep 53 bits above the last digit
@@ -91,12 +92,14 @@ def test_product_with_the_identity_is_exact(rt, n, bsize, spread):
     assert (np.abs(T.real - H) <= 2.0 ** -69 * largest).all()
 
 
+@pytest.mark.parametrize("most", [13, 4])
 @pytest.mark.parametrize("n,spacing", [(1, 1.0), (3, 1.0), (9, 1.0), (20, 0.5), (70, 0.1)])
-def test_series_and_sandwich_against_dense_algebra(rt, n, spacing):
-    """U and K' = U K U^dagger from random decaying blocks (1 to 70 triples an item; r = 6)."""
+def test_series_and_sandwich_against_dense_algebra(rt, n, spacing, most):
+    """U and K' = U K U^dagger from random decaying blocks (1 to 70 triples an item; r = 6; 4-function
+    systems with and without a last group of fewer than four atoms)."""
     rng = np.random.default_rng(n)
-    bsize = rng.integers(1, 14, size=n)
-    bsize[0] = 13
+    bsize = rng.integers(1, most + 1, size=n)
+    bsize[0] = most
     raw = {}
 
     def block(i, j):
