@@ -135,7 +135,7 @@ struct Sys {
 
 // Host copies: threads that share one large pageable copy, and the pinned piece of each
 constexpr int IO_THREADS = 8;
-constexpr size_t IO_PIECE = size_t(2) << 20;
+constexpr size_t IO_PIECE = size_t(512) << 10;
 
 // Grouped products of the reference split (one launch per product and block
 // size across all (system, kick) pairs) and their launch shapes
@@ -1883,7 +1883,7 @@ static void copy_host(rt_ctx* c, void* dst, const void* src, size_t bytes, bool 
   const bool known = cudaPointerGetAttributes(&at, to_host ? dst : src) == cudaSuccess;
   if (!known) cudaGetLastError();
   const bool pinned = known && at.type != cudaMemoryTypeUnregistered;
-  if (pinned || bytes < 2 * IO_PIECE) {
+  if (pinned || bytes < 2 * IO_THREADS * IO_PIECE) {
     if (bytes) RT_CUDA_CHECK(cudaMemcpyAsync(dst, src, bytes, kind, c->ws));
     RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
     return;
