@@ -416,27 +416,47 @@ static void reserve_split(rt_ctx* c, int n_atoms, int64_t nnzb_a, int64_t nnzb_b
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   RT_CUDA_CHECK(cudaStreamIsCapturing(c->ws, &cs));
   RT_REQUIRE(cs == cudaStreamCaptureStatusNone, RT_EINTERNAL, "split operands must be sized before a capture");
-  auto grow = [&](auto*& p, size_t& have, size_t want) {
-    if (want <= have) return;
-    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
-    using T = std::remove_reference_t<decltype(*p)>;
+  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+  c->graph_dirty = true;  // a captured step holds the old addresses
+  // a failed allocation leaves the sizes at zero: the next product asks again
+  auto give = [&](auto*& p) {
     if (p) c->arena.put(p);
     p = nullptr;
+  };
+  auto remake = [&](X64Operand& x, size_t& have, size_t want) {
+    if (want <= have) return;
     have = 0;
-    p = static_cast<T*>(c->arena.get(want));
+    give(x.dig);
+    give(x.lead);
+    x.dig = static_cast<unsigned char*>(c->arena.get(want));
+    x.lead = static_cast<unsigned char*>(c->arena.get(want / x64_block_bytes(false)));
     have = want;
   };
-  size_t la = c->xa_bytes / x64_block_bytes(false), lb = c->xb_bytes / x64_block_bytes(false);
-  grow(c->xa.lead, la, na / x64_block_bytes(false));
-  grow(c->xb.lead, lb, nb / x64_block_bytes(false));
-  grow(c->xa.dig, c->xa_bytes, na);
-  grow(c->xb.dig, c->xb_bytes, nb);
-  size_t ea = (size_t)c->x_atoms * 64, eb = ea;
-  const size_t ne = (size_t)std::max(n_atoms, c->x_atoms) * 64;
-  grow(c->xa.exps, ea, ne);
-  grow(c->xb.exps, eb, ne);
-  c->x_atoms = std::max(n_atoms, c->x_atoms);
-  c->graph_dirty = true;  // a captured step holds the old addresses
+  remake(c->xa, c->xa_bytes, na);
+  remake(c->xb, c->xb_bytes, nb);
+  if (n_atoms > c->x_atoms) {
+    c->x_atoms = 0;
+    give(c->xa.exps);
+    give(c->xb.exps);
+    c->xa.exps = c->arena.get_n<int32_t>((size_t)n_atoms * 16);
+    c->xb.exps = c->arena.get_n<int32_t>((size_t)n_atoms * 16);
+    c->x_atoms = n_atoms;
+  }
+}
+
+// The split operands of every product that a captured step may hold.
+static void reserve_for_step(rt_ctx* c, Sys& s) {
+  if (c->p.precision != RT_FP64) return;
+  int64_t most = 0;
+  if (s.B == 13) {
+    for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
+    reserve_split(c, s.n_atoms, most, most, true);
+  } else if (s.B == 4) {
+    for (const auto& q : s.qcache) most = std::max(most, q.second->P.nnzb);
+    bool any = false;
+    for (const auto& ti : s.tcache) any = any || ti.second->quads;
+    if (any) reserve_split(c, (s.n_atoms + 3) / 4, most, most, true);
+  }
 }
 
 // keep_a: A is the operand of the product just before, unchanged since, so that its split
@@ -779,19 +799,7 @@ static void setup_system(rt_ctx* c, Sys& s, const rt_system& in) {
       s.planar = p.packed_fma != 0 && !p.tensor_cores;
     }
   }
-  if (s.B == 13 && p.precision == RT_FP64) {
-    // the captured step holds FP64 products: their split operands are sized here
-    int64_t most = 0;
-    for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
-    reserve_split(c, s.n_atoms, most, most, true);
-  }
-  if (s.B == 4 && p.precision == RT_FP64) {
-    int64_t most = 0;
-    for (const auto& q : s.qcache) most = std::max(most, q.second->P.nnzb);
-    bool any = false;
-    for (const auto& ti : s.tcache) any = any || ti.second->quads;
-    if (any) reserve_split(c, (s.n_atoms + 3) / 4, most, most, true);
-  }
+  reserve_for_step(c, s);
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
 
@@ -2348,6 +2356,7 @@ rt_status rt_step(rt_ctx* c, int32_t n) {
       if (c->profiling) collect_profile(c);
     } else {
       if (c->graph_dirty || !c->gexec) {
+        for (auto& sp : c->sys) reserve_for_step(c, *sp);
         if (c->gexec) {
           cudaGraphExecDestroy(c->gexec);
           c->gexec = nullptr;
