@@ -216,11 +216,11 @@ inline int sb32(int B) { return B * rs32(B); }
 bool launch_gemm13_tc(Epilogue epi, const GemmArgs& g, cudaStream_t st);
 
 // FP64 products of 13-function atoms on the tensor cores (spgemm13_x64.cu): an
-// operand split into 64-bit fixed-point digits, one power-of-two scale per row
+// operand split into 72-bit fixed-point digits, one power-of-two scale per row
 // of op(A) / column of op(B), in the order in which a warp's registers take it.
 struct X64Operand {
   unsigned char* dig = nullptr;  // [nnzb][1 real, 2 complex][4096]
-  unsigned char* lead = nullptr; // [nnzb][1 real, 2 complex] leading digits that are zero in the whole block
+  unsigned char* lead = nullptr; // [nnzb][1 real, 2 complex] leading digits that are zero in the whole block (255: all)
   int32_t* exps = nullptr;       // [n_atoms][16] biased exponent of each scale
 };
 size_t x64_block_bytes(bool cplx);

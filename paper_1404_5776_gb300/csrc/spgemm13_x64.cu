@@ -5,52 +5,58 @@
 // list of the output block).  GB300 does two FP64 fused multiply-adds per clock
 // and SM, and the CUDA-core kernel ran at 87 % of that (a real triple: 1,099
 // clocks); the tensor cores do about a thousand FP16 ones through mma.sync.  So
-// every operand is written in 64-bit fixed point and multiplied digit by digit,
+// every operand is written in 72-bit fixed point and multiplied digit by digit,
 // exactly (the error-free splitting of Ozaki, Ogita, Oishi and Rump, Numer.
 // Algorithms 59, 2012):
 //   * each row of op(A) (each column of op(B)) takes one power-of-two scale,
 //     the first power 2^e above its magnitudes over the whole block row
 //     (column); each block takes off it the whole digits that its own largest
-//     value leaves at zero (z of them): x = X 2^(e - 8 z - 62), X an integer
-//     rounded to nearest, |X| < 2^62;
-//   * X in radix 256 with digits -128..127: the bytes of X + 0x8080..80 are the
-//     digits plus 128, so the split is one 64-bit addition;
-//   * a pair of digits (p, q) has the weight p + q + z_A + z_B; the pairs of
-//     weights 0..8 are multiplied as FP16 integers (one m16n8k16 per pair and
-//     8-column half: 43 pairs with z_A + z_B = 0, 28 with two, 15 with four),
-//     each weight in its own FP32 accumulators.  One triple adds an integer of at
-//     most 13 * 8 * 2^14 to a weight, so CARRY = 8 of them stay below 2^24 and
-//     are exact; then multiples of 256 move up one weight, exactly as well;
+//     value leaves at zero (z of them): x = X 2^(e - 9 z - 70), X an integer
+//     rounded to nearest, |X| < 2^70;
+//   * X in radix 512 with digits -256..255: the 9-bit groups of X + 256 (1 + 512 +
+//     ... + 512^7) are the digits plus 256, so the split is one addition;
+//   * a pair of digits (p, q) has the weight p + q + z_A + z_B; weights count from
+//     the first one that any triple of the item reaches, and the pairs of weights
+//     0..8 from there on are multiplied as FP16 integers (one m16n8k16 per pair and
+//     8-column half: 43 pairs for a triple that starts at the first, 28 two
+//     weights further, 15 four), each weight in its own FP32 accumulators.  These
+//     stay integers below 2^24 for CARRY products, and so exact; then multiples of
+//     512 move up one weight, exactly as well;
 //   * at the end the weights meet as two 64-bit integers, and these in FP64 with
 //     one rounding.
-// Measured against quad precision on the 64- and 216-atom cells (r = 6, 8,
-// 10 A; S^-1 H and U K U^dagger): relative 2-norm error 4e-17..8e-17, where FP64
-// fused multiply-adds gave 4e-16..4e-15; the median error of single elements is
-// 7e-17..7e-16 (3e-16..2e-15 before).
+// An entry keeps its 53 bits down to 2^-17 of the largest of its row (column) in a
+// near block, and is rounded to 2^-71 of the block's share of the scale below that;
+// what the pairs left out add is smaller still.  So the error of an element is
+// bounded by the scales of its row and column, not by its own terms as that of
+// multiply-adds is (n 2^-53 of |A||B|); on the library's matrices it is the smaller
+// of the two element by element, as the blocks' entries spread over far less than
+// the 2^18 between 2^-53 and 2^-71.  Measured over 64-bit-mantissa sums (64 and 216
+// atoms x 13, 512 x 4, r = 6..10 A), S^-1 H and U K U^dagger: relative 2-norm error 4e-17 to
+// 8e-17 (multiply-adds 4e-16 to 3e-15), the largest error of a single element over |A||B|
+// 6e-17 to 6e-16 (9e-16 to 8e-15).  (64 bits in radix 256, with the weights of an item
+// counted from its row's scale, are 10 % faster and leave up to 4e-13 there.)
 //
 // Layout: a split block is stored in the order in which an m16n8k16 operand
 // lies in a warp's registers (lane = 4 (row mod 8) + (k mod 8)/2), 16 bytes a
 // lane and load: one digit of op(A), two digits of one 8-column half of op(B).
 // Operands go from L2 straight into registers, without shared memory.  Rows and
-// k of 13..15 are padding.  One byte a digit (half the traffic, expanded in
-// registers) measured 1.03 times slower, the expansion being on the critical
-// path.
+// k of 13..15 are padding.
 //
 // One warp owns an 8-column half of a real output (a complex item: four warps,
 // halves x real and imaginary part, reading the same blocks through L1): 36
 // accumulators, 32 registers of A's digits and 16 of B's fit 128 registers, so
 // 16 warps a SM; a warp with both halves (168 registers, 12 warps) measured 1.3
-// times slower.  What bounds it: the tensor pipe (52-70 % busy in the Taylor
-// powers), with the wait for the next blocks' first digits beside it.
-// 216 atoms x 13, r = 8 A: a Taylor power 8.9 -> 1.14 ms with its splits, M = U K
-// 21.7 -> 3.3 ms; FP64 EM step at 512 atoms 126 -> 20.5 ms.  The time follows the
-// warps in flight: A's digits in two sets of registers (12 warps) took 27 % longer,
-// five CTAs of 96 registers (spills) 65 %.
+// times slower.  What bounds it: the tensor pipe, with the wait for the next blocks'
+// first digits and the carries beside it.  216 atoms x 13, r = 8 A: a Taylor power
+// 1.15 ms with its splits 1.20, M = U K 2.80 ms (the CUDA-core kernel: 8.9 and 21.7 ms);
+// FP64 EM step at 512 atoms 22 ms (126).  The time follows the warps in flight: A's
+// digits in two sets of registers (12 warps) took 27 % longer, five CTAs of 96
+// registers (spills) 65 %.
 //
 // 4-function atoms take the same kernel in quads: the blocks between two groups of
 // four consecutive atoms as one 16 x 16 block, absent ones zero (a 4 x 4 triple
 // alone would fill an eighth of a product).  FP64 EM step of 1728 atoms x 4 at 8 A:
-// 12.4 -> 7.0 ms; of 64 atoms x 4: 0.41 -> 0.18 ms.
+// 7.7 ms (one lane group a block on the CUDA cores: 12.4); of 64 atoms x 4: 0.16 ms (0.41).
 #include <algorithm>
 
 #include "rt_internal.cuh"
@@ -73,38 +79,55 @@ constexpr int MINB = 4;
 // warps of a CTA: an item takes 2 (real) or 4 (complex) for each share of its triples
 template <bool CPLX, int KS>
 constexpr int CTA_WARPS = (CPLX ? 4 : 2) * KS > WARPS ? (CPLX ? 4 : 2) * KS : WARPS;
-constexpr int NW = 9;          // weights p + q of the digit pairs that are multiplied
-// real products between two carries: (13 or 16) * 8 * 2^14 * CARRY + the carries < 2^24
-template <bool QUAD>
-constexpr int CARRY = QUAD ? 6 : 8;
+constexpr int NW = 9;          // weights of the digit pairs that are multiplied
+// real products between two carries: a weight has at most seven pairs of digits, of which the
+// first is at most 128, so that a product adds at most 16 * 7 * 2^16 to weights 4..8 and, with
+// up to four pairs, 16 * 3 * 2^16 to weights 0..3; with what the carries leave and bring in,
+// CARRY and 2 CARRY of them stay below 2^24
+constexpr int CARRY = 2;
+constexpr int HIGH = 4;        // weights below this one carry at every second turn
+constexpr int DIGIT = 9;       // bits of a digit
 constexpr int EXP_NAN = 2047;  // scale of a row that holds a NaN or an infinity: its products are NaN
-constexpr int MAX_LEAD = 9;    // a block with so many leading zero digits adds nothing (NW weights)
+constexpr int MAX_LEAD = 120;  // leading zero digits that a block's shift takes off at most
+constexpr int ZERO_LEAD = 255; // a block of zeros (above 2 MAX_LEAD + NW: no product of it has a weight)
 constexpr int SPLIT_WARPS = 16;
 
 // ---------------------------------------------------------------------------
 // split: one CTA per atom; its block row (by_col: its block column, reached
 // through the transposes) is read for the scales, then again (from L2) for the
-// digits.  Bound by the integer pipe that builds the digits (58 % busy): 30 us
-// for the 31 MB of a real matrix at 216 atoms, 3 % of the product that it serves.
+// digits.  Bound by the integer pipe that builds the digits: 52 us for the 31 MB
+// of a real matrix at 216 atoms, 5 % of the product that it serves.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long fixed_biased(double x, int ex_row) {
-  const unsigned long long bias = 0x8080808080808080ull;
+// x in 72-bit fixed point, 256 added to each digit: hi and lo hold four digits each.
+__device__ __forceinline__ void fixed_biased(double x, int ex_row, unsigned long long& hi, unsigned long long& lo) {
+  constexpr long long BIAS = 256ll * (1 + (1ll << 9) + (1ll << 18) + (1ll << 27)), MASK = (1ll << 36) - 1;
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int ex = (int)((b >> 52) & 0x7ff);
   unsigned long long m = b & 0xfffffffffffffull;
   if (ex) m |= 1ull << 52;
-  if (m == 0) return bias;
-  // |x| < 2^(ex_row - 1022); X = x 2^(62 - (ex_row - 1022)) = m 2^(max(ex,1) - ex_row + 9)
-  const int s = max(ex, 1) - ex_row + 9;
-  if (s >= 0) m <<= s;
-  else m = s > -64 ? (m + (1ull << (-s - 1))) >> -s : 0ull;
-  const unsigned long long v = (b >> 63) ? 0ull - m : m;
-  return v + bias;
+  // |x| < 2^(ex_row - 1022); X = x 2^(70 - (ex_row - 1022)) = m 2^(max(ex,1) - ex_row + 17)
+  int s = max(ex, 1) - ex_row + 17;
+  if (s < 0) {
+    m = s > -64 ? (m + (1ull << (-s - 1))) >> -s : 0ull;
+    s = 0;
+  }
+  long long h = (long long)(m >> (36 - s)), l = (long long)((m << s) & MASK);
+  if (b >> 63) {
+    h = -h;
+    l = -l;
+  }
+  l += BIAS;
+  hi = (unsigned long long)(h + BIAS + (l >> 36));
+  lo = (unsigned long long)(l & MASK);
 }
 
-__device__ __forceinline__ unsigned less_1152(unsigned h) {
+// Two biased digits (18 bits) as the FP16 numbers 1024 + u in the lower and upper half.
+__device__ __forceinline__ unsigned two_digits(unsigned w) {
+  return (w & 0x1ffu) | ((w << 7) & 0x1ff0000u) | 0x64006400u;
+}
+__device__ __forceinline__ unsigned less_1280(unsigned h) {
   unsigned r;
-  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x64806480u));
+  asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(h), "r"(0x65006500u));
   return r;
 }
 
@@ -135,7 +158,7 @@ struct SplitPair {
 };
 
 template <bool CPLX, bool QUAD>
-__global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const __grid_constant__ SplitPair pair) {
+__global__ void __launch_bounds__(SPLIT_WARPS * 32, 2) k_split13(const __grid_constant__ SplitPair pair) {
   const SplitArgs& s = pair.s[blockIdx.y];
   const double* __restrict__ vals = s.vals;
   const int32_t* __restrict__ map = s.map;
@@ -204,36 +227,31 @@ __global__ void __launch_bounds__(SPLIT_WARPS * 32) k_split13(const __grid_const
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       // the block's own shift: whole digits that its largest value leaves at zero, from the
-      // exponents alone (|x| < 2^(ex - 1022) and 2^62 is the row's bound)
-      int gap = 8 * MAX_LEAD;
+      // exponents alone (|x| < 2^(ex - 1022) and 2^70 is the row's bound)
+      int gap = DIGIT * ZERO_LEAD;
 #pragma unroll
       for (int f = 0; f < 8; ++f) {
         const int ex = (__double2hiint(val[c][f]) >> 20) & 0x7ff;
-        if (ex) gap = min(gap, smax[g + ((f >> 1) & 1) * 8] - ex);
+        if (val[c][f] != 0.0) gap = min(gap, smax[g + ((f >> 1) & 1) * 8] - max(ex, 1));
       }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) gap = min(gap, __shfl_xor_sync(0xffffffffu, gap, off));
-      const int z = gap >> 3;
+      gap = __reduce_min_sync(0xffffffffu, gap);
+      const int z = gap == DIGIT * ZERO_LEAD ? ZERO_LEAD : min(gap / DIGIT, MAX_LEAD);
       if (lane == 0) lead[(int64_t)qb * NC + c] = (unsigned char)z;
-      unsigned long long X[8];
+      unsigned long long X[8][2];  // digits 0..3 and 4..7
 #pragma unroll
       for (int f = 0; f < 8; ++f)
-        X[f] = fixed_biased(z < MAX_LEAD ? val[c][f] : 0.0, smax[g + ((f >> 1) & 1) * 8] - 8 * z);
+        fixed_biased(val[c][f], smax[g + ((f >> 1) & 1) * 8] - DIGIT * z, X[f][0], X[f][1]);
       uint4* out = reinterpret_cast<uint4*>(dig + ((int64_t)qb * NC + c) * BLK) + lane;
 #pragma unroll
       for (int p2 = 0; p2 < 4; ++p2) {  // digits 2 p2 and 2 p2 + 1, most significant first
         unsigned w[2][4];
 #pragma unroll
-        for (int d = 0; d < 2; ++d) {
-          const int p = 2 * p2 + d;
-#pragma unroll
-          for (int r = 0; r < 4; ++r) {
-            const unsigned lo = p < 4 ? (unsigned)(X[2 * r] >> 32) : (unsigned)X[2 * r];
-            const unsigned hi = p < 4 ? (unsigned)(X[2 * r + 1] >> 32) : (unsigned)X[2 * r + 1];
-            // the bytes uu of both, as the FP16 numbers 1024 + uu (0x64uu), less 1152
-            const unsigned two = __byte_perm(lo, hi, (3 - (p & 3)) | (7 - (p & 3)) << 4);  // bytes 0, 1
-            w[d][r] = less_1152(__byte_perm(two, 0x64646464u, 0x4140));
-          }
+        for (int r = 0; r < 4; ++r) {
+          const unsigned a = (unsigned)(X[2 * r][p2 >> 1] >> (p2 & 1 ? 0 : 18)) & 0x3ffffu;
+          const unsigned b = (unsigned)(X[2 * r + 1][p2 >> 1] >> (p2 & 1 ? 0 : 18)) & 0x3ffffu;
+          const unsigned ta = two_digits(a), tb = two_digits(b);
+          w[0][r] = less_1280(__byte_perm(ta, tb, 0x7632));
+          w[1][r] = less_1280(__byte_perm(ta, tb, 0x5410));
         }
         if (right) {
           // op(B): the 8-column halves apart, two digits of one half together
@@ -268,13 +286,32 @@ __device__ __forceinline__ void mma16816(float (&c)[4], const uint4& a, unsigned
       : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
       : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
-// v 2^(ea - 1022) 2^(eb - 1022), a normal result by its exponent field alone; a
-// row with a NaN or an infinity gives NaN
-__device__ __forceinline__ double pow2_scaled(double v, int ea, int eb) {
+// v 2^(ea - 1022) 2^(eb - 1022) 2^-shift, a normal result by its exponent field
+// alone; a row with a NaN or an infinity gives NaN
+__device__ __forceinline__ double pow2_scaled(double v, int ea, int eb, int shift) {
   if (ea == EXP_NAN || eb == EXP_NAN) return __longlong_as_double(0x7ff8000000000000ll);
-  const int k = ea + eb - 2044, h = __double2hiint(v), ex = ((h >> 20) & 0x7ff) + k;
+  const int k = ea + eb - 2044 - shift, h = __double2hiint(v), ex = ((h >> 20) & 0x7ff) + k;
   if (v == 0.0) return 0.0;
   return ex > 0 && ex < 2047 ? __hiloint2double(h + k * (1 << 20), __double2loint(v)) : ldexp(v, k);
+}
+// pairs of FP32 numbers in one register pair
+__device__ __forceinline__ unsigned long long pair_of(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpair(unsigned long long v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
 }
 // an FP32 integer below 2^22 in magnitude
 __device__ __forceinline__ int small_int(float v) { return __float_as_int(v + 12582912.f) - 0x4b400000; }
@@ -342,31 +379,32 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
 #pragma unroll
     for (int w = 0; w < NW; ++w) acc[w][r] = 0.f;
   }
-  // moves multiples of 256 up one weight (FP32 integers below 2^24: every operation is exact)
-  auto carry = [&] {
+  // moves multiples of 512 up one weight, from the last weight to `first` (FP32 integers below
+  // 2^24: every operation is exact; two at a time, a third of the warp's issue slots otherwise)
+  auto carry = [&](int first, int last) {
     constexpr float MAGIC = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer
+    const unsigned long long part512 = pair_of(1.f / 512.f, 1.f / 512.f), minus512 = pair_of(-512.f, -512.f);
+    const unsigned long long plus = pair_of(MAGIC, MAGIC), minus = pair_of(-MAGIC, -MAGIC);
 #pragma unroll
     for (int w = NW - 1; w >= 0; --w)
+      if (w >= first && w <= last) {
+        float(&up)[4] = w > 0 ? acc[w > 0 ? w - 1 : 0] : top;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float c = __fadd_rn(__fmaf_rn(acc[w][r], 1.f / 256.f, MAGIC), -MAGIC);
-        acc[w][r] = __fmaf_rn(c, -256.f, acc[w][r]);
-        if (w > 0) acc[w - 1][r] += c;
-        else top[r] += c;
+        for (int r = 0; r < 4; r += 2) {
+          const unsigned long long v = pair_of(acc[w][r], acc[w][r + 1]);
+          const unsigned long long c = add2(fma2(v, part512, plus), minus);
+          unpair(fma2(c, minus512, v), acc[w][r], acc[w][r + 1]);
+          unpair(add2(pair_of(up[r], up[r + 1]), c), up[r], up[r + 1]);
+        }
       }
   };
 
   const int64_t t0 = g.ptr[item];
   int nt = (int)(g.ptr[item + 1] - t0);
   const int2* __restrict__ ab = g.ab + t0;
-  if constexpr (KS > 1) {  // this warp's share of the triples
-    const int share = (nt + KS - 1) / KS, first = min(nt, share * ks);
-    ab += first;
-    nt = min(share, nt - first);
-  }
   const unsigned char* __restrict__ dA = x.dA + lane * 16;
   const unsigned char* __restrict__ dB = x.dB + lane * 16 + half * (BLK / 2);
-  // digits to skip of a triple's blocks: bytes 0, 1: A's parts, bytes 2, 3: B's
+  // leading zero digits of a triple's blocks: bytes 0, 1: A's parts, bytes 2, 3: B's
   auto leads = [&](int2 p) {
     if constexpr (CPLX)
       return (unsigned)reinterpret_cast<const unsigned short*>(x.lA)[p.x] |
@@ -376,6 +414,20 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
   };
   auto lead_a = [&](unsigned z, int sub) { return (int)((z >> (8 * sub)) & 0xff); };
   auto lead_b = [&](unsigned z, int sub) { return (int)((z >> (16 + 8 * (CPLX ? (sub ^ part) : 0))) & 0xff); };
+  // weights count from the first that any triple of the item (of all its shares) reaches:
+  // a far block keeps as many digits of its own as a near one
+  int z0 = ZERO_LEAD;
+  for (int t = lane; t < nt; t += 32) {
+    const unsigned z = leads(ab[t]);
+#pragma unroll
+    for (int sub = 0; sub < NP; ++sub) z0 = min(z0, lead_a(z, sub) + lead_b(z, sub));
+  }
+  z0 = __reduce_min_sync(0xffffffffu, z0);
+  if constexpr (KS > 1) {  // this warp's share of the triples
+    const int share = (nt + KS - 1) / KS, first = min(nt, share * ks);
+    ab += first;
+    nt = min(share, nt - first);
+  }
   if (nt > 0) {
     // triples t, t + 1 and t + 2 of the list; the digits to skip of the first two
     int2 cur = ab[0], nxt = 1 < nt ? ab[1] : cur, nxt2 = 2 < nt ? ab[2] : nxt;
@@ -403,7 +455,7 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
         const uint4* na = reinterpret_cast<const uint4*>(dA + ((int64_t)nb.x * NP + ns) * BLK);
         const uint4* nbp = reinterpret_cast<const uint4*>(dB + ((int64_t)nb.y * NP + (CPLX ? (ns ^ part) : 0)) * BLK);
         // weights below the first that can be non-zero, of this product and the next
-        const int zz = lead_a(zc, sub) + lead_b(zc, sub), znext = lead_a(z, ns) + lead_b(z, ns);
+        const int zz = lead_a(zc, sub) + lead_b(zc, sub) - z0, znext = lead_a(z, ns) + lead_b(z, ns) - z0;
         if (CPLX && (sub ? neg1 : neg0)) {
 #pragma unroll
           for (int p = 0; p < 8; ++p) {
@@ -429,8 +481,10 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
           case 8: multiply<8, !CPLX>(acc, a, b, na, nbp, znext); break;
           default: multiply<NW, !CPLX>(acc, a, b, na, nbp, znext); break;  // below every weight: nothing but the loads
         }
-        if (++since == CARRY<QUAD>) {
-          carry();
+        ++since;
+        if (since % CARRY == 0) carry(HIGH, NW - 1);
+        if (since == 2 * CARRY) {
+          carry(0, HIGH - 1);
           since = 0;
         }
       }
@@ -440,21 +494,21 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
       zc = zn;
       zn = zn2;
     }
-    carry();
+    carry(0, NW - 1);
   }
 
   const int q = g.item_blk[item];
   const int i = g.rowidx[q], j = g.colidx[q];
-  // the weights as two integers, hi 2^48 + lo in units of 256^6 2^-124
+  // the weights as two integers, hi 2^54 + lo in units of 512^6 2^-140
   long long hi[4], lo[4];
 #pragma unroll
   for (int rr = 0; rr < 4; ++rr) {
-    const int lo1 = (small_int(acc[3][rr]) * 256 + small_int(acc[4][rr])) * 256 + small_int(acc[5][rr]);
-    const int lo0 = (small_int(acc[6][rr]) * 256 + small_int(acc[7][rr])) * 256 + small_int(acc[8][rr]);
+    const int lo1 = (small_int(acc[3][rr]) * 512 + small_int(acc[4][rr])) * 512 + small_int(acc[5][rr]);
+    const int lo0 = (small_int(acc[6][rr]) * 512 + small_int(acc[7][rr])) * 512 + small_int(acc[8][rr]);
     const int hi1 = __float2int_rn(top[rr]);
-    const int hi0 = (small_int(acc[0][rr]) * 256 + small_int(acc[1][rr])) * 256 + small_int(acc[2][rr]);
-    lo[rr] = (long long)lo1 * (1 << 24) + lo0;
-    hi[rr] = (long long)hi1 * (1 << 24) + hi0;
+    const int hi0 = (small_int(acc[0][rr]) * 512 + small_int(acc[1][rr])) * 512 + small_int(acc[2][rr]);
+    lo[rr] = (long long)lo1 * (1 << 27) + lo0;
+    hi[rr] = (long long)hi1 * (1 << 27) + hi0;
   }
   if constexpr (KS > 1) {
     const int base = warp % WPB;
@@ -480,11 +534,16 @@ __global__ void __launch_bounds__(CTA_WARPS<CPLX, KS> * 32, MINB * WARPS / CTA_W
     for (int rr = 0; rr < 4; ++rr) {
       const int r = gr + (rr >> 1) * 8, c = 8 * half + 2 * tc + (rr & 1);
       if (r < BS && c < BS) {
-        // the integers enter FP64 as mantissas of 1.5 2^24 and 1.5 2^-24 (exact), and meet with one rounding
-        constexpr double MH = 0x1.8p24, ML = 0x1.8p-24;
-        const double vh = __longlong_as_double(__double_as_longlong(MH) + hi[rr]) - MH;
-        const double vl = __longlong_as_double(__double_as_longlong(ML) + lo[rr]) - ML;
-        sC[slot][(r * BS + c) * NP + part] = pow2_scaled(vh + vl, x.eA[i * 16 + r], x.eB[j * 16 + c]);
+        // lo within 2^53, so that it is exact in FP64; the integers enter as mantissas of 1.5 2^20,
+        // 1.5 2^-7 and 1.5 2^-34 (exact), and the two halves of lo, then hi and lo meet: one rounding
+        const long long up = (lo[rr] + (1ll << 53)) >> 54;
+        const long long l = lo[rr] - (up << 54), l0 = ((l + (1ll << 26)) & ((1ll << 27) - 1)) - (1ll << 26);
+        constexpr double MH = 0x1.8p20, M1 = 0x1.8p-7, M0 = 0x1.8p-34;
+        const double vh = __longlong_as_double(__double_as_longlong(MH) + hi[rr] + up) - MH;
+        const double v1 = __longlong_as_double(__double_as_longlong(M1) + ((l - l0) >> 27)) - M1;
+        const double v0 = __longlong_as_double(__double_as_longlong(M0) + l0) - M0;
+        sC[slot][(r * BS + c) * NP + part] =
+            pow2_scaled(vh + (v1 + v0), x.eA[i * 16 + r], x.eB[j * 16 + c], DIGIT * z0);
       }
     }
   }
