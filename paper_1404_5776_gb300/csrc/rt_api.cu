@@ -460,21 +460,26 @@ static void reserve_for_step(rt_ctx* c, Sys& s) {
 }
 
 // keep_a: A is the operand of the product just before, unchanged since, so that its split
-// stands (if that product took the same route, which xa_of says)
+// stands (if that product took the same route, which xa_of says).
+// quads: off for products of propagators with one another.  Beside its diagonal of ones a
+// propagator falls by up to 2^25 within a quad (216 and 512 atoms x 4, Si:H clusters; 8 to 10 A),
+// and where both operands do, 1 to 15 in 1000 far elements of the product lose up to 2e-13 of
+// |A||B|, where multiply-adds lose 4e-15; with a density or a power of T on one side none does.
 static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cplx, bool ad, bool bd, Epilogue epi,
-                 GemmArgs g, const Pattern* C, bool keep_a = false) {
+                 GemmArgs g, const Pattern* C, bool keep_a = false, bool quads = true) {
   g = prepared(c, s, ti, fp32, cplx, epi, g, C);
   int B = s.B;
   const Pattern* had = c->xa_of;
   c->xa_of = nullptr;
-  if ((B == 13 && c->p.precision == RT_FP64) || ti.quads) {
+  quads = quads && ti.quads;
+  if ((B == 13 && c->p.precision == RT_FP64) || quads) {
     // products of the FP64 mode: exact digit products on the tensor cores, of 13-function blocks (6x
     // the CUDA cores at every size measured, 64 to 512 atoms) and of quads of 4-function blocks;
     // the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
-    const Pattern &pa = ti.quads ? ti.qa->P : *ti.pa, &pb = ti.quads ? ti.qb->P : *ti.pb;
-    const int32_t *ma = ti.quads ? ti.qa->map : nullptr, *mb = ti.quads ? ti.qb->map : nullptr,
-                  *mc = ti.quads ? ti.qc->map : nullptr;
-    if (ti.quads) {
+    const Pattern &pa = quads ? ti.qa->P : *ti.pa, &pb = quads ? ti.qb->P : *ti.pb;
+    const int32_t *ma = quads ? ti.qa->map : nullptr, *mb = quads ? ti.qb->map : nullptr,
+                  *mc = quads ? ti.qc->map : nullptr;
+    if (quads) {
       g.item_blk = ti.qt.item_blk;
       g.ptr = ti.qt.ptr;
       g.ab = ti.qt.ab;
@@ -991,7 +996,7 @@ static void build_etrs(rt_ctx* c, Sys& s, bool fp32) {
   field_T(c, s, E_TDT, s.T);
   taylor_series(c, s, s.T, 0.5 * p.dt, p.taylor_terms, false, s.Xn);
   TripleInfo& tUU = triples_for(c, s, s.pU, false, s.pU, false, s.pU, false);
-  gemm(c, s, PC_TAYLOR, tUU, false, true, false, false, EPI_STORE, args(s.Xn, s.X, s.U), s.pU);
+  gemm(c, s, PC_TAYLOR, tUU, false, true, false, false, EPI_STORE, args(s.Xn, s.X, s.U), s.pU, false, false);
 }
 
 // fourth-order Magnus (Sec. II.A): T1, T2 at t + (1/2 -+ sqrt(3)/6) dt,
@@ -1838,11 +1843,11 @@ static void unitarity(rt_ctx* c, Sys& s, int metric, double* mx, double* mean) {
   if (metric) {
     TripleInfo& tW = triples_for(c, s, s.pS, false, s.pU, false, s.pW, false);
     TripleInfo& tE = triples_for(c, s, s.pU, true, s.pW, false, s.pU, false);
-    gemm(c, s, PC_MISC, tW, false, true, false, false, EPI_STORE, args(s.Sc, s.U, s.W), s.pW);
-    gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.W, s.E), s.pU);
+    gemm(c, s, PC_MISC, tW, false, true, false, false, EPI_STORE, args(s.Sc, s.U, s.W), s.pW, false, false);
+    gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.W, s.E), s.pU, false, false);
   } else {
     TripleInfo& tE = triples_for(c, s, s.pU, true, s.pU, false, s.pU, false);
-    gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.U, s.E), s.pU);
+    gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.U, s.E), s.pU, false, false);
   }
   double* pmax = c->arena.get_n<double>(1024);
   double* psum = c->arena.get_n<double>(1024);

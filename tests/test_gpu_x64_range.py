@@ -153,3 +153,77 @@ def test_entries_that_are_not_finite_stay_in_their_column(rt, b, n, bad):
     other = np.arange(b * n) != b + 2
     assert np.array_equal(T[:, other], H[:, other])
     assert not np.isfinite(T[:, b + 2]).any()  # 0 * inf and inf reach every row, as in multiply-adds
+
+
+@pytest.mark.parametrize("cell,radius", [(3, 8.0), (4, 6.0)])
+def test_product_of_two_propagators(rt, cell, radius):
+    """ETRS without a field: U = cut(V V), V the EM propagator of half the step.  Every element within seven standard
+    deviations of n roundings of |V||V| (2 sqrt(n) 2^-53), also where V falls by 2^20 among four neighbouring atoms."""
+    import synth
+    s = synth.diamond_system(cell, "sp4", 6.0, 6.0, seed=0)
+    radii = {k: radius for k in RADII}
+    got = []
+    for prop, dt in (("etrs", 0.05), ("em", 0.025)):
+        ctx = rt.RT(s, prop=prop, dt=dt, **radii)
+        ctx.inverse()
+        ctx.propagator(0.0)
+        rowptr, col = ctx.pattern(0, rt.RT_PAT_U)
+        near = np.zeros((s.n_atoms, s.n_atoms), bool)
+        near[np.repeat(np.arange(s.n_atoms), np.diff(rowptr)), col] = True
+        got.append(_dense(ctx.matrix(0, rt.RT_MAT_U), near, 4))
+        ctx.close()
+    U, V = got
+    rows = np.arange(0, 4 * s.n_atoms, 37)
+    cut = np.kron(near, np.ones((4, 4)))[rows]
+    re, im = V.real.astype(np.longdouble), V.imag.astype(np.longdouble)
+    exact_re, exact_im = re[rows] @ re - im[rows] @ im, re[rows] @ im + im[rows] @ re
+    a, b = np.abs(V.real), np.abs(V.imag)
+    n = 2 * 4 * near.sum(1).max()
+    bound = 2.0 * np.sqrt(n) * 2.0 ** -53
+    for part, exact, terms in ((U.real, exact_re, a[rows] @ a + b[rows] @ b), (U.imag, exact_im, a[rows] @ b + b[rows] @ a)):
+        err = np.abs(part[rows] - exact * cut).astype(float)
+        assert (err <= bound * terms * cut).all(), (err / np.where(terms > 0, terms, 1.0)).max()
+
+
+@pytest.mark.parametrize("which,power", [(range(13), 0), (range(8, 13), 1), (range(8, 13), -1), (range(12, 13), -3), (range(0, 1), -2)])
+def test_scaled_basis_functions(rt, which, power):
+    """Some functions of every atom times 2^power, as far as the inverse's stopping rule goes along (2^2 up, 2^-5 down and
+    it reports a stagnated residual): S^-1 H from the library's own S^-1, and one step's K' = U K U^dagger from its own U,
+    every element within seven standard deviations of n roundings of the terms' absolute values."""
+    import synth
+    s = synth.diamond_system(2, "spd13", 7.0, 7.0, seed=0)
+    n = 13 * s.n_atoms
+    f = np.ones(13)
+    f[list(which)] = 2.0 ** power
+    outer = np.outer(f, f).reshape(-1)
+    scale = lambda v: (v.reshape(-1, 169) * outer).reshape(-1)
+    s = dataclasses.replace(s, s_val=scale(s.s_val), h_val=scale(s.h_val), d_val=[scale(d) for d in s.d_val])
+    radii = {k: 8.0 for k in RADII}
+    ctx = rt.RT(s, prop="em", dt=0.05, **radii)
+    ctx.inverse()
+    rowptr, col = ctx.pattern(0, rt.RT_PAT_U)
+    near = np.zeros((s.n_atoms, s.n_atoms), bool)
+    near[np.repeat(np.arange(s.n_atoms), np.diff(rowptr)), col] = True
+    cut = np.kron(near, np.ones((13, 13))).astype(bool)
+    rng = np.random.default_rng(1)
+    K0 = rng.normal(size=(n, n)) + 1j * rng.normal(size=(n, n))
+    K0 = (K0 + K0.conj().T) * cut / np.outer(np.tile(f, s.n_atoms), np.tile(f, s.n_atoms))
+    ctx.set_density_dense(0, 0, K0)
+    ctx.step(1)
+    X, T, U, K = (_dense(ctx.matrix(0, m), near, 13) for m in (rt.RT_MAT_SINV, rt.RT_MAT_T, rt.RT_MAT_U, rt.RT_MAT_K))
+    ctx.close()
+    H, X, T = s.to_dense("H"), X.real, T.real
+    rows = np.arange(0, n, 61)
+    q = np.longdouble
+    roundings = 2.0 * np.sqrt(n) * 2.0 ** -53
+    err = np.abs(T[rows] - (X[rows].astype(q) @ H.astype(q)) * cut[rows]).astype(float)
+    assert (err <= roundings * (np.abs(X[rows]) @ np.abs(H)) * cut[rows]).all()
+    parts = lambda a: (a.real.astype(q), a.imag.astype(q))
+    (ur, ui), (kr, ki), (vr, vi) = parts(U[rows]), parts(K0), parts(U)
+    mr, mi = (ur @ kr - ui @ ki) * cut[rows], (ur @ ki + ui @ kr) * cut[rows]
+    exact = (mr @ vr.T + mi @ vi.T) + 1j * (mi @ vr.T - mr @ vi.T)
+    atom = np.arange(n) // 13
+    up = cut[rows] & (atom[None, :] > atom[rows][:, None])
+    terms = ((np.abs(U[rows]) @ np.abs(K0)) * cut[rows]) @ np.abs(U).T
+    err = np.abs((K[rows] - exact).astype(complex))
+    assert (err <= 4.0 * roundings * terms)[up].all()
