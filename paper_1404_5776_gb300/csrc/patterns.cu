@@ -16,18 +16,23 @@ namespace rt {
 // memory
 // ----------------------------------------------------------------------------
 void* Allocator::get(size_t bytes, cudaStream_t stream) {
-  void* p = nullptr;
-  if (alloc) {
-    p = alloc(bytes, (void*)stream, user);
-    RT_REQUIRE(p != nullptr, RT_ENOMEM, "allocator hook returned NULL for " + std::to_string(bytes) + " bytes");
-  } else {
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      throw Error{RT_ENOMEM, "cudaMalloc(" + std::to_string(bytes) + ") failed: " + cudaGetErrorString(e)};
+  for (;;) {
+    void* p = nullptr;
+    std::string why;
+    if (alloc) {
+      p = alloc(bytes, (void*)stream, user);
+      if (!p) why = "allocator hook returned NULL for " + std::to_string(bytes) + " bytes";
+    } else {
+      const cudaError_t e = cudaMalloc(&p, bytes);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+        why = "cudaMalloc(" + std::to_string(bytes) + ") failed: " + cudaGetErrorString(e);
+      }
     }
+    if (p) return p;
+    if (!spare || !spare()) throw Error{RT_ENOMEM, why};
   }
-  return p;
 }
 
 void Allocator::put(void* p, cudaStream_t stream) {
@@ -41,7 +46,6 @@ void* Arena::get(size_t bytes) {
   if (bytes == 0) bytes = 256;
   void* p = alloc->get(bytes, stream);
   blocks.push_back(p);
-  total += bytes;
   return p;
 }
 
@@ -57,7 +61,6 @@ void Arena::put(void* p) {
 void Arena::release_all() {
   for (void* p : blocks) alloc->put(p, stream);
   blocks.clear();
-  total = 0;
 }
 
 // ----------------------------------------------------------------------------

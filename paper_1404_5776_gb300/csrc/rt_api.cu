@@ -178,6 +178,7 @@ struct rt_ctx {
   size_t xa_bytes = 0, xb_bytes = 0;
   const rt::Pattern* xa_of = nullptr;  // pattern of the operand in xa after a product that split it
   int x_atoms = 0;
+  bool x_off = false;  // their memory was refused, or handed back to another request
   // pinned staging of host copies to and from pageable memory (made by the first large one)
   void* stage = nullptr;
   cudaEvent_t stage_ev[rt::IO_THREADS] = {};
@@ -409,39 +410,78 @@ static GemmArgs prepared(rt_ctx* c, Sys& s, TripleInfo& ti, bool fp32, bool cplx
   return g;
 }
 
-// Room for the split operands of a product over patterns of at most nnzb blocks.
-static void reserve_split(rt_ctx* c, int n_atoms, int64_t nnzb_a, int64_t nnzb_b, bool cplx) {
+// Hands the split operands' memory back: the products of this context stay on the CUDA cores from
+// here on (spgemm.cu), which need none.  False where there is nothing to hand back, or while a step
+// is being captured.
+static bool drop_split(rt_ctx* c) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (!c->ws || cudaStreamIsCapturing(c->ws, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+  bool any = false;
+  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+  auto give = [&](auto*& p) {
+    if (!p) return;
+    c->arena.put(p);
+    p = nullptr;
+    any = true;
+  };
+  for (X64Operand* x : {&c->xa, &c->xb}) {
+    give(x->dig);
+    give(x->lead);
+    give(x->exps);
+  }
+  c->xa_bytes = c->xb_bytes = 0;
+  c->x_atoms = 0;
+  c->xa_of = nullptr;
+  c->x_off = true;
+  c->graph_dirty = true;  // a captured step holds the addresses
+  return any;
+}
+
+// Room for the split operands of a product over patterns of at most nnzb blocks; false where the
+// allocator refused it, now or before.
+static bool room_for_split(rt_ctx* c, int n_atoms, int64_t nnzb_a, int64_t nnzb_b, bool cplx) {
+  if (c->x_off) return false;
   const size_t na = (size_t)nnzb_a * x64_block_bytes(cplx), nb = (size_t)nnzb_b * x64_block_bytes(cplx);
-  if (na <= c->xa_bytes && nb <= c->xb_bytes && n_atoms <= c->x_atoms) return;
+  if (na <= c->xa_bytes && nb <= c->xb_bytes && n_atoms <= c->x_atoms) return true;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   RT_CUDA_CHECK(cudaStreamIsCapturing(c->ws, &cs));
   RT_REQUIRE(cs == cudaStreamCaptureStatusNone, RT_EINTERNAL, "split operands must be sized before a capture");
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
   c->graph_dirty = true;  // a captured step holds the old addresses
-  // a failed allocation leaves the sizes at zero: the next product asks again
   auto give = [&](auto*& p) {
     if (p) c->arena.put(p);
     p = nullptr;
+  };
+  // a refusal hands the buffers made so far back (Allocator::spare), and the retry is not taken
+  auto make = [&](auto*& p, size_t n) {
+    if (!c->x_off) p = c->arena.get_n<std::remove_pointer_t<std::remove_reference_t<decltype(p)>>>(n);
   };
   auto remake = [&](X64Operand& x, size_t& have, size_t want) {
     if (want <= have) return;
     have = 0;
     give(x.dig);
     give(x.lead);
-    x.dig = static_cast<unsigned char*>(c->arena.get(want));
-    x.lead = static_cast<unsigned char*>(c->arena.get(want / x64_block_bytes(false)));
+    make(x.dig, want);
+    make(x.lead, want / x64_block_bytes(false));
     have = want;
   };
-  remake(c->xa, c->xa_bytes, na);
-  remake(c->xb, c->xb_bytes, nb);
-  if (n_atoms > c->x_atoms) {
-    c->x_atoms = 0;
-    give(c->xa.exps);
-    give(c->xb.exps);
-    c->xa.exps = c->arena.get_n<int32_t>((size_t)n_atoms * 16);
-    c->xb.exps = c->arena.get_n<int32_t>((size_t)n_atoms * 16);
-    c->x_atoms = n_atoms;
+  try {
+    remake(c->xa, c->xa_bytes, na);
+    remake(c->xb, c->xb_bytes, nb);
+    if (n_atoms > c->x_atoms) {
+      c->x_atoms = 0;
+      give(c->xa.exps);
+      give(c->xb.exps);
+      make(c->xa.exps, (size_t)n_atoms * 16);
+      make(c->xb.exps, (size_t)n_atoms * 16);
+      c->x_atoms = n_atoms;
+    }
+  } catch (const Error& e) {
+    if (e.code != RT_ENOMEM) throw;
+    c->x_off = true;
   }
+  if (c->x_off) drop_split(c);
+  return !c->x_off;
 }
 
 // The split operands of every product that a captured step may hold.
@@ -450,14 +490,17 @@ static void reserve_for_step(rt_ctx* c, Sys& s) {
   int64_t most = 0;
   if (s.B == 13) {
     for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
-    reserve_split(c, s.n_atoms, most, most, true);
+    room_for_split(c, s.n_atoms, most, most, true);
   } else if (s.B == 4) {
     for (const auto& q : s.qcache) most = std::max(most, q.second->P.nnzb);
     bool any = false;
     for (const auto& ti : s.tcache) any = any || ti.second->quads;
-    if (any) reserve_split(c, (s.n_atoms + 3) / 4, most, most, true);
+    if (any) room_for_split(c, (s.n_atoms + 3) / 4, most, most, true);
   }
 }
+
+// Whether a product with this triple list takes its quads
+static bool in_quads(const rt_ctx* c, const TripleInfo& ti) { return ti.quads && !c->x_off; }
 
 // keep_a: A is the operand of the product just before, unchanged since, so that its split
 // stands (if that product took the same route, which xa_of says).
@@ -471,12 +514,13 @@ static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cpl
   int B = s.B;
   const Pattern* had = c->xa_of;
   c->xa_of = nullptr;
-  quads = quads && ti.quads;
-  if ((B == 13 && c->p.precision == RT_FP64) || quads) {
+  quads = quads && in_quads(c, ti);
+  const Pattern &pa = quads ? ti.qa->P : *ti.pa, &pb = quads ? ti.qb->P : *ti.pb;
+  const bool digits = (B == 13 && c->p.precision == RT_FP64) || quads;
+  if (digits && (c->counting ? !c->x_off : room_for_split(c, pa.n_atoms, pa.nnzb, pb.nnzb, cplx))) {
     // products of the FP64 mode: exact digit products on the tensor cores, of 13-function blocks (6x
     // the CUDA cores at every size measured, 64 to 512 atoms) and of quads of 4-function blocks;
     // the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
-    const Pattern &pa = quads ? ti.qa->P : *ti.pa, &pb = quads ? ti.qb->P : *ti.pb;
     const int32_t *ma = quads ? ti.qa->map : nullptr, *mb = quads ? ti.qb->map : nullptr,
                   *mc = quads ? ti.qc->map : nullptr;
     if (quads) {
@@ -487,7 +531,6 @@ static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cpl
       g.rowidx = ti.qc->P.rowidx;
       g.colidx = ti.qc->P.col;
     }
-    if (!c->counting) reserve_split(c, pa.n_atoms, pa.nnzb, pb.nnzb, cplx);
     keep_a = keep_a && had == &pa;
     c->xa_of = &pa;
     run(
@@ -552,7 +595,7 @@ static GemmArgs args(const void* A, const void* B, void* C) {
 static void residual_from_items(rt_ctx* c, Sys& s, const TripleInfo& ti, double* out, double* out2) {
   run(
       c, PC_MISC, 0, 0,
-      [&] { launch_sum(s.red_items, ti.quads ? ti.qt.n_items : ti.t.n_items, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
+      [&] { launch_sum(s.red_items, in_quads(c, ti) ? ti.qt.n_items : ti.t.n_items, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
 }
 
 // ----------------------------------------------------------------------------
@@ -2068,6 +2111,7 @@ rt_status rt_create(rt_ctx** out, const rt_system* sys, int32_t n_sys, const rt_
   c->alloc.alloc = alloc;
   c->alloc.free = free_fn;
   c->alloc.user = alloc_user;
+  c->alloc.spare = [c] { return drop_split(c); };
   c->arena.alloc = &c->alloc;
   c->user = (cudaStream_t)cuda_stream;
   try {

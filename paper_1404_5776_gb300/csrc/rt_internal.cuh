@@ -16,6 +16,7 @@
 #include <stdint.h>
 #include <stdio.h>
 
+#include <functional>
 #include <string>
 #include <vector>
 
@@ -52,6 +53,7 @@ struct Allocator {
   rt_alloc_fn alloc = nullptr;
   rt_free_fn free = nullptr;
   void* user = nullptr;
+  std::function<bool()> spare;  // hands memory back when a request is refused; false: there is none
   void* get(size_t bytes, cudaStream_t stream);
   void put(void* p, cudaStream_t stream);
 };
@@ -61,7 +63,6 @@ struct Arena {
   Allocator* alloc = nullptr;
   cudaStream_t stream = nullptr;
   std::vector<void*> blocks;
-  size_t total = 0;
   void* get(size_t bytes);
   void put(void* p);  // gives one buffer back (the stream is done with it)
   template <typename T>
