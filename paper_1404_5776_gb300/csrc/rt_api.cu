@@ -11,8 +11,11 @@
 //   Tr(K S), Tr(K D_xyz) recorded per step.
 // All work runs on an internal stream ordered against the caller's stream with
 // events; a step is captured once in a CUDA graph and replayed.
+#include <unistd.h>
+
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstddef>
 #include <cstring>
@@ -133,9 +136,10 @@ struct Sys {
   std::string sinv_status;
 };
 
-// Host copies: threads that share one large pageable copy, and the pinned piece of each
+// Host copies: threads that share the first touch of a large buffer's pages, the chunk that one takes at a time, and
+// the size from which on they do
 constexpr int IO_THREADS = 8;
-constexpr size_t IO_PIECE = size_t(512) << 10;
+constexpr size_t IO_CHUNK = size_t(2) << 20, IO_TOUCH = size_t(8) << 20;
 
 // Grouped products of the reference split (one launch per product and block
 // size across all (system, kick) pairs) and their launch shapes
@@ -179,9 +183,6 @@ struct rt_ctx {
   const rt::Pattern* xa_of = nullptr;  // pattern of the operand in xa after a product that split it
   int x_atoms = 0;
   bool x_off = false;  // their memory was refused, or handed back to another request
-  // pinned staging of host copies to and from pageable memory (made by the first large one)
-  void* stage = nullptr;
-  cudaEvent_t stage_ev[rt::IO_THREADS] = {};
   void* zero32 = nullptr;  // one zero FP32 complex block (padded layout)
   int* d_err = nullptr;    // device error word of bounded waits
   long long wait_ns = 2000000000ll;  // budget of one bounded device wait
@@ -1928,59 +1929,46 @@ static Pattern* pattern_by_id(Sys& s, int which) {
   }
 }
 
-// Copies between the device and caller memory and waits.  A pinned buffer takes
-// one DMA.  Pageable memory of some size goes through pinned pieces, one per
-// thread: the host side of such a copy is bound by one core's memcpy and by the
-// first touch of the caller's pages, which the threads share (K of 512 atoms x 13
-// at 8 A, 148 MB into a new array: 25 -> 8 ms with the rest of the read).
-static void copy_host(rt_ctx* c, void* dst, const void* src, size_t bytes, bool to_host) {
-  const cudaMemcpyKind kind = to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice;
-  cudaPointerAttributes at{};
-  const bool known = cudaPointerGetAttributes(&at, to_host ? dst : src) == cudaSuccess;
-  if (!known) cudaGetLastError();
-  const bool pinned = known && at.type != cudaMemoryTypeUnregistered;
-  if (pinned || bytes < 2 * IO_THREADS * IO_PIECE) {
-    if (bytes) RT_CUDA_CHECK(cudaMemcpyAsync(dst, src, bytes, kind, c->ws));
-    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
-    return;
+// First touch of the pages of caller memory that a copy is about to fill: its time is one core's, clearing them
+// (148 MB: 4.5 of the copy's 5.3 ms), so IO_THREADS share the range, chunk by chunk.  The caller waits for chunks that
+// were taken and not for threads that have not run yet (on busy cores that is a time slice each); those find no chunk left
+// and touch nothing.  (A byte of each page is written without reading it: a read maps the shared page of zeros, and taking
+// that back from the device's translations costs 20 us a page.)
+struct PageTouch {
+  char* base;
+  size_t bytes, page;
+  std::atomic<size_t> next{0}, done{0};
+  size_t chunks() const { return (bytes + IO_CHUNK - 1) / IO_CHUNK; }
+  void take() {
+    for (size_t k; (k = next.fetch_add(1)) < chunks(); done.fetch_add(1))
+      for (size_t o = k * IO_CHUNK; o < std::min(bytes, (k + 1) * IO_CHUNK); o += page)
+        *const_cast<volatile char*>(base + o) = 0;
   }
-  if (!c->stage) {
-    for (cudaEvent_t& e : c->stage_ev)
-      if (!e) RT_CUDA_CHECK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-    RT_CUDA_CHECK(cudaMallocHost(&c->stage, IO_THREADS * IO_PIECE));
-  }
-  int dev = 0;
-  RT_CUDA_CHECK(cudaGetDevice(&dev));
-  const size_t pieces = (bytes + IO_PIECE - 1) / IO_PIECE;
-  const int n = (int)std::min<size_t>(IO_THREADS, pieces);
-  cudaError_t errs[IO_THREADS] = {};
-  // thread w moves the pieces w, w + n, ... through its own buffer; the copies of
-  // all threads follow one another on the context's stream
-  auto work = [&](int w) {
-    cudaError_t e = cudaSetDevice(dev);
-    char* buf = static_cast<char*>(c->stage) + (size_t)w * IO_PIECE;
-    for (size_t k = w; k < pieces && e == cudaSuccess; k += n) {
-      const size_t off = k * IO_PIECE, nb = std::min(IO_PIECE, bytes - off);
-      char* d = static_cast<char*>(dst) + off;
-      const char* s = static_cast<const char*>(src) + off;
-      if (!to_host) memcpy(buf, s, nb);
-      e = cudaMemcpyAsync(to_host ? buf : d, to_host ? s : buf, nb, kind, c->ws);
-      if (e == cudaSuccess) e = cudaEventRecord(c->stage_ev[w], c->ws);
-      if (e == cudaSuccess) e = cudaEventSynchronize(c->stage_ev[w]);
-      if (e == cudaSuccess && to_host) memcpy(d, buf, nb);
-    }
-    errs[w] = e;
-  };
-  std::vector<std::thread> pool;
-  int started = 1;
+};
+static void touch_pages(void* p, size_t bytes) {
+  auto t = std::make_shared<PageTouch>();
+  t->base = static_cast<char*>(p);
+  t->bytes = bytes;
+  t->page = (size_t)sysconf(_SC_PAGESIZE);
   try {
-    for (; started < n; ++started) pool.emplace_back(work, started);
-  } catch (...) {  // no more threads to be had: this one takes their pieces
+    for (int w = 1; w < IO_THREADS; ++w) std::thread([t] { t->take(); }).detach();
+  } catch (...) {  // no more threads to be had
   }
-  work(0);
-  for (std::thread& t : pool) t.join();
-  for (int w = started; w < n; ++w) work(w);
-  for (int w = 0; w < n; ++w) RT_CUDA_CHECK(errs[w]);
+  t->take();
+  while (t->done.load() < t->chunks()) std::this_thread::yield();
+}
+
+// Copies between the device and caller memory, pinned or not, and waits.  The device reaches pageable memory of the
+// Grace host itself, at 180 GB/s (148 MB: 0.7 to 0.8 ms; through pinned pieces 2.6), once its pages are there.
+static void copy_host(rt_ctx* c, void* dst, const void* src, size_t bytes, bool to_host) {
+  if (to_host && bytes >= IO_TOUCH) {
+    cudaPointerAttributes at{};
+    const bool known = cudaPointerGetAttributes(&at, dst) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (!known || at.type == cudaMemoryTypeUnregistered) touch_pages(dst, bytes);
+  }
+  if (bytes)
+    RT_CUDA_CHECK(cudaMemcpyAsync(dst, src, bytes, to_host ? cudaMemcpyDeviceToHost : cudaMemcpyHostToDevice, c->ws));
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
 
@@ -2833,9 +2821,6 @@ void rt_destroy(rt_ctx* c) {
     cudaEventDestroy(e.second);
   }
   c->arena.release_all();
-  if (c->stage) cudaFreeHost(c->stage);
-  for (cudaEvent_t e : c->stage_ev)
-    if (e) cudaEventDestroy(e);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ws) cudaStreamDestroy(c->ws);
