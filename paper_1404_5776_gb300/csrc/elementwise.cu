@@ -1131,24 +1131,24 @@ void launch_field_poly(const PolyTerms& V, int deg, const DevState* s, int which
 
 // ---------------------------------------------------------------------------
 // the caller's layout (true block sizes, complex) and padded device blocks; a
-// warp per block, off = first true element of each block (null: no padding)
+// warp per block, off = first true element of each block (null: no padding), `base` that of the first one
 // ---------------------------------------------------------------------------
-__global__ void k_pack_true(const double* __restrict__ v, int cplx, const int64_t* __restrict__ off, int64_t nnzb,
-                            const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
+__global__ void k_pack_true(const double* __restrict__ v, int cplx, const int64_t* __restrict__ off, int64_t base,
+                            int64_t nnzb, const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
                             const int32_t* __restrict__ bsize, int B, double2* __restrict__ out) {
   const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int NE = B * B;
   for (int64_t q = (int64_t)blockIdx.x * warps + (threadIdx.x >> 5); q < nnzb; q += (int64_t)gridDim.x * warps) {
     const int bi = off ? bsize[rowidx[q]] : B, bj = off ? bsize[col[q]] : B;
-    const int64_t o = off ? off[q] : q * NE;
+    const int64_t o = off ? off[q] - base : q * NE;
     for (int e = lane; e < bi * bj; e += 32) {
       const int64_t p = q * NE + (e / bj) * B + e % bj;
       out[o + e] = cplx ? reinterpret_cast<const double2*>(v)[p] : make_double2(v[p], 0.0);
     }
   }
 }
-__global__ void k_unpack_true(const double2* __restrict__ in, const int64_t* __restrict__ off, int64_t nnzb,
-                              const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
+__global__ void k_unpack_true(const double2* __restrict__ in, const int64_t* __restrict__ off, int64_t base,
+                              int64_t nnzb, const int32_t* __restrict__ rowidx, const int32_t* __restrict__ col,
                               const int32_t* __restrict__ bsize, int B, double2* __restrict__ v) {
   const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
   const int NE = B * B;
@@ -1156,22 +1156,22 @@ __global__ void k_unpack_true(const double2* __restrict__ in, const int64_t* __r
     const int bi = bsize[rowidx[q]], bj = bsize[col[q]];
     for (int e = lane; e < NE; e += 32) {
       const int a = e / B, b = e - a * B;
-      v[q * NE + e] = a < bi && b < bj ? in[off[q] + a * bj + b] : make_double2(0.0, 0.0);
+      v[q * NE + e] = a < bi && b < bj ? in[off[q] - base + a * bj + b] : make_double2(0.0, 0.0);
     }
   }
 }
 static unsigned pack_grid(int64_t nnzb) { return (unsigned)std::min<int64_t>((nnzb + 7) / 8, 152 * 32); }
-void launch_pack_true(const void* v, bool cplx, const int64_t* off, int64_t nnzb, const int32_t* rowidx,
+void launch_pack_true(const void* v, bool cplx, const int64_t* off, int64_t base, int64_t nnzb, const int32_t* rowidx,
                       const int32_t* col, const int32_t* bsize, int B, double2* out, cudaStream_t st) {
   if (nnzb == 0) return;
-  k_pack_true<<<pack_grid(nnzb), 256, 0, st>>>(static_cast<const double*>(v), cplx, off, nnzb, rowidx, col, bsize, B,
-                                               out);
+  k_pack_true<<<pack_grid(nnzb), 256, 0, st>>>(static_cast<const double*>(v), cplx, off, base, nnzb, rowidx, col,
+                                               bsize, B, out);
   RT_CUDA_CHECK(cudaGetLastError());
 }
-void launch_unpack_true(const double2* in, const int64_t* off, int64_t nnzb, const int32_t* rowidx, const int32_t* col,
-                        const int32_t* bsize, int B, double2* v, cudaStream_t st) {
+void launch_unpack_true(const double2* in, const int64_t* off, int64_t base, int64_t nnzb, const int32_t* rowidx,
+                        const int32_t* col, const int32_t* bsize, int B, double2* v, cudaStream_t st) {
   if (nnzb == 0) return;
-  k_unpack_true<<<pack_grid(nnzb), 256, 0, st>>>(in, off, nnzb, rowidx, col, bsize, B, v);
+  k_unpack_true<<<pack_grid(nnzb), 256, 0, st>>>(in, off, base, nnzb, rowidx, col, bsize, B, v);
   RT_CUDA_CHECK(cudaGetLastError());
 }
 

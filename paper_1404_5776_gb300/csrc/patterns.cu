@@ -15,7 +15,7 @@ namespace rt {
 // ----------------------------------------------------------------------------
 // memory
 // ----------------------------------------------------------------------------
-void* Allocator::get(size_t bytes, cudaStream_t stream) {
+void* Allocator::get(size_t bytes, cudaStream_t stream, bool use_spare) {
   for (;;) {
     void* p = nullptr;
     std::string why;
@@ -31,7 +31,7 @@ void* Allocator::get(size_t bytes, cudaStream_t stream) {
       }
     }
     if (p) return p;
-    if (!spare || !spare()) throw Error{RT_ENOMEM, why};
+    if (!use_spare || !spare || !spare()) throw Error{RT_ENOMEM, why};
   }
 }
 
@@ -41,10 +41,10 @@ void Allocator::put(void* p, cudaStream_t stream) {
   else cudaFree(p);
 }
 
-void* Arena::get(size_t bytes) {
+void* Arena::get(size_t bytes, bool use_spare) {
   bytes = (bytes + 255) & ~size_t(255);
   if (bytes == 0) bytes = 256;
-  void* p = alloc->get(bytes, stream);
+  void* p = alloc->get(bytes, stream, use_spare);
   blocks.push_back(p);
   return p;
 }

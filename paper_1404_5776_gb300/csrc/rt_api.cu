@@ -77,7 +77,12 @@ struct Sys {
           *pM = nullptr, *pA = nullptr, *pW = nullptr;
   std::map<double, std::unique_ptr<Pattern>> pcache;
   std::unique_ptr<Pattern> pS_given, pH_given;
-  std::map<const Pattern*, int64_t*> true_off;  // padded systems: first true element of each block (device)
+  // padded systems: first true element of each block in the caller's layout, and their number at the end
+  struct TrueOffsets {
+    std::vector<int64_t> h;
+    int64_t* d = nullptr;
+  };
+  std::map<const Pattern*, TrueOffsets> true_off;
   std::map<TripleKey, std::unique_ptr<TripleInfo>> tcache;
   std::map<const Pattern*, std::unique_ptr<QuadPattern>> qcache;
   // FP64 values (padded blocks)
@@ -140,6 +145,7 @@ struct Sys {
 // the size from which on they do
 constexpr int IO_THREADS = 8;
 constexpr size_t IO_CHUNK = size_t(2) << 20, IO_TOUCH = size_t(8) << 20;
+constexpr size_t IO_BUFFER = size_t(64) << 20;  // device memory that a read or write may pack blocks in
 
 // Grouped products of the reference split (one launch per product and block
 // size across all (system, kick) pairs) and their launch shapes
@@ -571,8 +577,8 @@ struct Scratch {
   std::vector<void*> ptrs;
   explicit Scratch(rt_ctx* ctx) : c(ctx) {}
   template <typename T>
-  T* get_n(size_t n) {
-    void* p = c->alloc.get(n * sizeof(T) + 16, c->ws);
+  T* get_n(size_t n, bool use_spare = true) {
+    void* p = c->alloc.get(n * sizeof(T) + 16, c->ws, use_spare);
     ptrs.push_back(p);
     return static_cast<T*>(p);
   }
@@ -1972,25 +1978,87 @@ static void copy_host(rt_ctx* c, void* dst, const void* src, size_t bytes, bool 
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
 
-// First true element of each block of P in the caller's layout (padded systems; device)
-static const int64_t* true_offsets(rt_ctx* c, Sys& s, const Pattern* P) {
-  auto it = s.true_off.find(P);
-  if (it != s.true_off.end()) return it->second;
-  std::vector<int64_t> off(P->nnzb);
-  int64_t n = 0;
-  for (int i = 0; i < s.n_atoms; ++i)
-    for (int q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
-      off[q] = n;
-      n += (int64_t)s.bsize[i] * s.bsize[P->h_col[q]];
+static const Sys::TrueOffsets& true_offsets(rt_ctx* c, Sys& s, const Pattern* P) {
+  Sys::TrueOffsets& off = s.true_off[P];
+  if (off.h.empty()) {
+    off.h.reserve(P->nnzb + 1);
+    int64_t n = 0;
+    for (int i = 0; i < s.n_atoms; ++i)
+      for (int q = P->h_rowptr[i]; q < P->h_rowptr[i + 1]; ++q) {
+        off.h.push_back(n);
+        n += (int64_t)s.bsize[i] * s.bsize[P->h_col[q]];
+      }
+    off.h.push_back(n);
+  }
+  if (!off.d) {  // stays null where the device has no room for it
+    try {
+      off.d = static_cast<int64_t*>(c->arena.get(sizeof(int64_t) * off.h.size(), false));
+    } catch (const Error& e) {
+      if (e.code != RT_ENOMEM) throw;
+      return off;
     }
-  int64_t* d = c->arena.get_n<int64_t>(off.size());
-  if (!off.empty())
-    RT_CUDA_CHECK(cudaMemcpyAsync(d, off.data(), sizeof(int64_t) * off.size(), cudaMemcpyHostToDevice, c->ws));
-  RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
-  s.true_off[P] = d;
-  return d;
+    RT_CUDA_CHECK(cudaMemcpyAsync(off.d, off.h.data(), sizeof(int64_t) * off.h.size(), cudaMemcpyHostToDevice, c->ws));
+    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+  }
+  return off;
 }
 static bool padded(const Sys& s) { return s.n_true != (int64_t)s.n_atoms * s.B; }
+
+// Blocks of P between the device's layout (dev: padded, real or complex) and the caller's (host: true sizes, complex),
+// a stretch of them at a time: in a buffer of at most IO_BUFFER on the device, packed there, or, where there is no room for
+// one, on the host.  (A read or write is not worth the split operands: the buffer is asked for without the allocator's spare.)
+static void copy_blocks(rt_ctx* c, Sys& s, const Pattern* P, double* dev, bool cplx, double* host, bool to_host) {
+  const int B = s.B, NE = B * B, parts = cplx ? 2 : 1;
+  const bool pad = padded(s);
+  const Sys::TrueOffsets* off = pad ? &true_offsets(c, s, P) : nullptr;
+  auto first = [&](int64_t q) { return off ? off->h[q] : q * NE; };
+  const int64_t per = std::max<int64_t>(1, std::min<int64_t>(P->nnzb, IO_BUFFER / (sizeof(double2) * NE)));
+  std::vector<double> blocks;
+  Scratch tmp(c);
+  double2* packed = nullptr;
+  if (!pad || off->d) {
+    try {
+      packed = tmp.get_n<double2>(per * NE, false);
+    } catch (const Error& e) {
+      if (e.code != RT_ENOMEM) throw;
+    }
+  }
+  if (!packed) blocks.resize((size_t)std::min<int64_t>(per, IO_CHUNK / (sizeof(double2) * NE)) * NE * parts);
+  const int64_t step = packed ? per : (int64_t)blocks.size() / (NE * parts);
+  int i = 0;  // row of block q (host packing)
+  for (int64_t q0 = 0; q0 < P->nnzb; q0 += step) {
+    const int64_t q1 = std::min(P->nnzb, q0 + step), n = q1 - q0;
+    const size_t bytes = sizeof(double2) * (size_t)(first(q1) - first(q0));
+    double *d = dev + q0 * NE * parts, *h = host + 2 * first(q0);
+    if (packed) {
+      const int64_t* d_off = pad ? off->d + q0 : nullptr;
+      if (to_host)
+        launch_pack_true(d, cplx, d_off, first(q0), n, P->rowidx + q0, P->col + q0, s.d_bsize, B, packed, c->ws);
+      copy_host(c, to_host ? (void*)h : packed, to_host ? (const void*)packed : h, bytes, to_host);
+      if (!to_host) {
+        launch_unpack_true(packed, d_off, first(q0), n, P->rowidx + q0, P->col + q0, s.d_bsize, B,
+                           reinterpret_cast<double2*>(d), c->ws);
+        RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+      }
+      continue;
+    }
+    if (to_host) copy_host(c, blocks.data(), d, sizeof(double) * n * NE * parts, true);
+    else std::fill(blocks.begin(), blocks.end(), 0.0);
+    for (int64_t q = q0; q < q1; ++q) {
+      while (q >= P->h_rowptr[i + 1]) ++i;
+      const int bi = s.bsize[i], bj = s.bsize[P->h_col[q]];
+      double* blk = blocks.data() + (q - q0) * NE * parts;
+      for (int a = 0; a < bi; ++a)
+        for (int b = 0; b < bj; ++b, h += 2)
+          for (int k = 0; k < 2; ++k) {
+            double* e = blk + (a * B + b) * parts + k;
+            if (!to_host) *e = h[k];
+            else h[k] = k < parts ? *e : 0.0;
+          }
+    }
+    if (!to_host) copy_host(c, d, blocks.data(), sizeof(double) * n * NE * parts, false);
+  }
+}
 
 // (pattern, device values, complex?) of a readable matrix
 static void matrix_by_id(rt_ctx* c, Sys& s, int kick, int which, Pattern** P, const void** v, bool* cplx) {
@@ -2226,8 +2294,6 @@ rt_status rt_set_density(rt_ctx* c, int32_t sys, int32_t kick, const double* h) 
     RT_REQUIRE(kick >= 0 && kick < c->p.n_kick, RT_EINVAL, "kick index out of range");
     RT_REQUIRE(h, RT_EINVAL, "NULL density");
     Sys& s = *c->sys[sys];
-    const Pattern& P = *s.pK;
-    const int B = s.B;
     // K replaced: it is the density again; the reference split keeps K_ref and
     // carries the new K as dK = K - K_ref from the next step
     if (!s.dk_fresh.empty()) s.dk_fresh[kick] = 0;
@@ -2238,13 +2304,8 @@ rt_status rt_set_density(rt_ctx* c, int32_t sys, int32_t kick, const double* h) 
       copy_host(c, s.K[kick], h, sizeof(double2) * nvals(s, s.pK), false);
       return RT_OK;
     }
-    const int64_t n = true_elems(s, &P);
-    Scratch tmp(c);
-    double2* compact = tmp.get_n<double2>(n);
     reset_time(c);
-    copy_host(c, compact, h, sizeof(double2) * n, false);
-    launch_unpack_true(compact, true_offsets(c, s, &P), P.nnzb, P.rowidx, P.col, s.d_bsize, B, s.K[kick], c->ws);
-    RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
+    copy_blocks(c, s, s.pK, reinterpret_cast<double*>(s.K[kick]), true, const_cast<double*>(h), false);
     return RT_OK;
   });
 }
@@ -2517,11 +2578,7 @@ rt_status rt_get_matrix(rt_ctx* c, int32_t sys, int32_t kick, int32_t which, dou
       copy_host(c, vals, v, sizeof(double) * need, true);
       return RT_OK;
     }
-    Scratch tmp(c);
-    double2* compact = tmp.get_n<double2>(need / 2);
-    launch_pack_true(v, cplx, padded(s) ? true_offsets(c, s, P) : nullptr, P->nnzb, P->rowidx, P->col, s.d_bsize, s.B,
-                     compact, c->ws);
-    copy_host(c, vals, compact, sizeof(double) * need, true);
+    copy_blocks(c, s, P, static_cast<double*>(const_cast<void*>(v)), cplx, vals, true);
     return RT_OK;
   });
 }

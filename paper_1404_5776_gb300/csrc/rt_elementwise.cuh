@@ -129,10 +129,10 @@ void launch_u_from_delta(const float2* dU, double2* U, int64_t nnzb, const int32
 void launch_u_minus_i_f32(const double2* U, float2* dU, int64_t nnzb, const int32_t* rowidx, const int32_t* col,
                           int B, cudaStream_t st);
 
-// Padded device blocks to the caller's layout (complex, true sizes) and back; off as in k_pack_true.
-void launch_pack_true(const void* v, bool cplx, const int64_t* off, int64_t nnzb, const int32_t* rowidx,
+// Padded device blocks to the caller's layout (complex, true sizes) and back; off and base as in k_pack_true.
+void launch_pack_true(const void* v, bool cplx, const int64_t* off, int64_t base, int64_t nnzb, const int32_t* rowidx,
                       const int32_t* col, const int32_t* bsize, int B, double2* out, cudaStream_t st);
-void launch_unpack_true(const double2* in, const int64_t* off, int64_t nnzb, const int32_t* rowidx, const int32_t* col,
-                        const int32_t* bsize, int B, double2* v, cudaStream_t st);
+void launch_unpack_true(const double2* in, const int64_t* off, int64_t base, int64_t nnzb, const int32_t* rowidx,
+                        const int32_t* col, const int32_t* bsize, int B, double2* v, cudaStream_t st);
 
 }  // namespace rt

@@ -54,7 +54,7 @@ struct Allocator {
   rt_free_fn free = nullptr;
   void* user = nullptr;
   std::function<bool()> spare;  // hands memory back when a request is refused; false: there is none
-  void* get(size_t bytes, cudaStream_t stream);
+  void* get(size_t bytes, cudaStream_t stream, bool use_spare = true);
   void put(void* p, cudaStream_t stream);
 };
 
@@ -63,7 +63,7 @@ struct Arena {
   Allocator* alloc = nullptr;
   cudaStream_t stream = nullptr;
   std::vector<void*> blocks;
-  void* get(size_t bytes);
+  void* get(size_t bytes, bool use_spare = true);
   void put(void* p);  // gives one buffer back (the stream is done with it)
   template <typename T>
   T* get_n(size_t n) {

@@ -1,5 +1,5 @@
-"""Densities, matrices and states of more than 8 MB in pageable memory: they come back as they went in, and a copy takes
-about the time of one plain copy of that size."""
+"""Densities, matrices and states of more than 8 MB in pageable memory: they come back as they went in, also where the
+device has no memory to spare, and a copy takes about the time of one plain copy of that size."""
 import time
 
 import numpy as np
@@ -72,4 +72,30 @@ def test_a_pageable_density_is_set_at_the_rate_of_a_plain_copy(rt):
 
     copy = best(lambda: plain.copy_(torch.from_numpy(K)))
     assert best(lambda: ctx.set_density(0, 0, K)) <= 2.0 * copy
+    ctx.close()
+
+
+# 13 functions (real matrices packed), 1 and 4 functions (all packed)
+@pytest.mark.parametrize("system,precision", [("diamond", "fp64"), ("diamond", "fp32"), ("cluster", "fp64")])
+def test_matrices_are_read_and_set_without_device_memory_to_spare(rt, monkeypatch, system, precision):
+    from test_gpu_memory import Limited
+    s = synth.diamond_system(2, "spd13", 6.0, 6.0, seed=0) if system == "diamond" else _cluster(150)
+    mem = Limited(rt)
+    monkeypatch.setattr(rt, "_torch_allocator", lambda: mem.hooks)
+    ctx = rt.RT(s, prop="em", dt=0.05, precision=precision, **_radii(8.0))
+    ctx.inverse()
+    K = _values(rt, ctx, s, np.random.default_rng(0))
+    ctx.set_density(0, 0, K)
+    read = lambda: [ctx.matrix(0, m) for m in (rt.RT_MAT_SINV, rt.RT_MAT_T, rt.RT_MAT_K)]
+    ctx.step(1)
+    before, held = read(), dict(mem.held)
+    mem.limit = mem.now
+    for got, want in zip(read(), before):
+        assert np.array_equal(got, want)
+    ctx.set_density(0, 0, K)
+    assert np.array_equal(ctx.matrix(0, rt.RT_MAT_K), K)
+    ctx.step(1)
+    mem.limit = None
+    assert np.array_equal(ctx.matrix(0, rt.RT_MAT_K), before[2])
+    assert mem.held == held  # the split operands among it
     ctx.close()
