@@ -601,7 +601,7 @@ int64_t triple_true_macs(const Triples& T, const Pattern& A, bool a_dag, const P
 
 // Host pass over the rows of one group at a time: the groups that its atoms
 // reach, ascending, and the blocks of each.
-void build_quads(QuadPattern& Q, const Pattern& P, Arena& arena, cudaStream_t st) {
+void build_quads(QuadPattern& Q, const Pattern& P, cudaStream_t st) {
   const int n = P.n_atoms, m = (n + 3) / 4;
   std::vector<int32_t> rowptr(m + 1, 0), col, map, seen(m, -1), cols;
   for (int I = 0; I < m; ++I) {
@@ -627,8 +627,8 @@ void build_quads(QuadPattern& Q, const Pattern& P, Arena& arena, cudaStream_t st
     for (int J : cols) seen[J] = -1;
     rowptr[I + 1] = (int32_t)col.size();
   }
-  upload_pattern(Q.P, m, rowptr.data(), col.data(), P.radius, arena, st);
-  Q.map = arena.get_n<int32_t>(map.size());
+  upload_pattern(Q.P, m, rowptr.data(), col.data(), P.radius, Q.mem, st);
+  Q.map = Q.mem.get_n<int32_t>(map.size());
   if (!map.empty())
     RT_CUDA_CHECK(cudaMemcpyAsync(Q.map, map.data(), sizeof(int32_t) * map.size(), cudaMemcpyHostToDevice, st));
   RT_CUDA_CHECK(cudaStreamSynchronize(st));

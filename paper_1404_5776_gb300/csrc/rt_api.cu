@@ -22,6 +22,7 @@
 #include <limits>
 #include <map>
 #include <memory>
+#include <set>
 #include <thread>
 #include <tuple>
 
@@ -51,11 +52,12 @@ struct TripleKey {
 struct TripleInfo {
   const Pattern *pa = nullptr, *pb = nullptr;  // the operands' patterns
   Triples t;
-  // FP64 4-function products as quads (16 x 16 blocks of four consecutive atoms): the quads'
-  // list and patterns; taken where `quads`
+  // FP64 4-function products as quads (16 x 16 blocks of four consecutive atoms): triples to a product of quads,
+  // and, where that is enough for either kind of product, the quads' list and patterns
+  double quad_fill = 0.0;
+  bool quads_counted = false;
   Triples qt;
   const QuadPattern *qa = nullptr, *qb = nullptr, *qc = nullptr;
-  bool quads = false;
   TileList tiles;  // row tiles for the tensor-core kernel (built for the sandwich's FP32 13-function products)
   int64_t true_macs = 0;
   int64_t nnzb_a = 0, nnzb_b = 0;
@@ -290,17 +292,86 @@ static Pattern* pattern_for(rt_ctx* c, Sys& s, double r) {
   return raw;
 }
 
-// Quads are taken from this many 4-function triples to a product of quads on:
-// one of 16 x 16 (exact digits on the tensor cores, spgemm13_x64.cu) measured as
-// long as 6.7 real or 5.0 complex 4-function triples on the FP64 pipe (1728 atoms:
-// 0.82 against 0.122 ns, 2.3 against 0.46 ns).  In lattice order there are 9 to 11
-// of them at 8 A, 4.7 at 6 A, 61 in a 64-atom cell.
-constexpr int QUAD_FILL = 6;
+// Quads are taken from this many 4-function triples to a product of quads on, a real or a complex one: there the
+// product of 16 x 16 blocks (exact digits on the tensor cores, spgemm13_x64.cu) takes as long as its triples on the FP64
+// pipe.  Measured over 216, 512 and 1728 atoms at 6 to 9 A (quads / FP64 pipe, us): Taylor power 137 / 100 at 4.5 triples,
+// 269 / 256 at 6.6, 198 / 192 at 7.3, 573 / 582 at 7.7, 641 / 806 at 7.8, 298 / 372 at 8.8; M = U K 389 / 303 at 4.9,
+// 447 / 464 at 5.9, 839 / 935 at 6.6, 578 / 683 at 7.3.
+constexpr double QUAD_FILL_REAL = 7.5, QUAD_FILL_CPLX = 5.75;
 
-static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* B, bool bd, Pattern* C, bool up) {
+// The quads of a triple list, where there are triples enough to a product of them.  Patterns that no list takes are given
+// back by release_quads.
+static void add_quads(rt_ctx* c, Sys& s, TripleInfo& ti, const TripleKey& k) {
+  ti.quads_counted = true;
+  auto quad = [&](const Pattern* P) {
+    std::unique_ptr<QuadPattern>& Q = s.qcache[P];
+    if (!Q) {
+      auto made = std::make_unique<QuadPattern>();
+      made->mem.alloc = &c->alloc;
+      made->mem.stream = c->ws;
+      try {
+        build_quads(*made, *P, c->ws);
+      } catch (...) {
+        cudaStreamSynchronize(c->ws);
+        made->mem.release_all();
+        throw;
+      }
+      Q = std::move(made);
+    }
+    return Q.get();
+  };
+  const QuadPattern *qa, *qb, *qc;
+  Arena list;
+  list.alloc = &c->alloc;
+  list.stream = c->ws;
+  Triples qt;
+  try {
+    qa = quad(k.A);
+    qb = quad(k.B);
+    qc = quad(k.C);
+    build_triples(qt, qa->P, k.ad, qb->P, k.bd, qc->P, k.up, list, c->ws);
+  } catch (const Error& e) {
+    list.release_all();
+    if (e.code != RT_ENOMEM) throw;
+    return;  // no memory for them: the CUDA-core products need none
+  }
+  const double fill = qt.n_triples ? (double)ti.t.n_triples / (double)qt.n_triples : 0.0;
+  if (fill < std::min(QUAD_FILL_REAL, QUAD_FILL_CPLX)) {
+    list.release_all();
+    return;
+  }
+  c->arena.blocks.insert(c->arena.blocks.end(), list.blocks.begin(), list.blocks.end());
+  ti.quad_fill = fill;
+  ti.qt = qt;
+  ti.qa = qa;
+  ti.qb = qb;
+  ti.qc = qc;
+}
+
+static void release_quads(Sys& s) {
+  std::set<const QuadPattern*> used;
+  for (const auto& kv : s.tcache)
+    for (const QuadPattern* Q : {kv.second->qa, kv.second->qb, kv.second->qc}) used.insert(Q);
+  for (auto it = s.qcache.begin(); it != s.qcache.end();) {
+    if (it->second && used.count(it->second.get())) {
+      ++it;
+      continue;
+    }
+    if (it->second) it->second->mem.release_all();
+    it = s.qcache.erase(it);
+  }
+}
+
+// quads: off for products that do not take them (gemm)
+static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* B, bool bd, Pattern* C, bool up,
+                               bool quads = true) {
   TripleKey key{A, B, C, ad, bd, up};
+  quads = quads && s.B == 4 && c->p.precision == RT_FP64;
   auto it = s.tcache.find(key);
-  if (it != s.tcache.end()) return *it->second;
+  if (it != s.tcache.end()) {
+    if (quads && !it->second->quads_counted) add_quads(c, s, *it->second, key);
+    return *it->second;
+  }
   auto ti = std::make_unique<TripleInfo>();
   build_triples(ti->t, *A, ad, *B, bd, *C, up, c->arena, c->ws);
   ti->true_macs = triple_true_macs(ti->t, *A, ad, *C, s.d_bsize, c->arena, c->ws);
@@ -329,25 +400,11 @@ static TripleInfo& triples_for(rt_ctx* c, Sys& s, Pattern* A, bool ad, Pattern* 
     for (int32_t q : items) n += (int64_t)s.bsize[rowof[q]] * s.bsize[C->h_col[q]];
     ti->true_elems_c = n;
   }
-  if (s.B == 4 && c->p.precision == RT_FP64) {
-    auto quad = [&](Pattern* P) {
-      std::unique_ptr<QuadPattern>& Q = s.qcache[P];
-      if (!Q) {
-        Q = std::make_unique<QuadPattern>();
-        build_quads(*Q, *P, c->arena, c->ws);
-      }
-      return Q.get();
-    };
-    ti->qa = quad(A);
-    ti->qb = quad(B);
-    ti->qc = quad(C);
-    build_triples(ti->qt, ti->qa->P, ad, ti->qb->P, bd, ti->qc->P, up, c->arena, c->ws);
-    ti->quads = ti->t.n_triples >= (int64_t)QUAD_FILL * ti->qt.n_triples;
-  }
   if (ti->t.n_items > s.red_items_n) {
     s.red_items = c->arena.get_n<double>(ti->t.n_items);
     s.red_items_n = ti->t.n_items;
   }
+  if (quads) add_quads(c, s, *ti, key);
   TripleInfo& ref = *ti;
   s.tcache[key] = std::move(ti);
   return ref;
@@ -499,15 +556,16 @@ static void reserve_for_step(rt_ctx* c, Sys& s) {
     for (const Pattern* P : {s.pS, s.pH, s.pSinv, s.pT, s.pU, s.pK, s.pM, s.pA}) most = std::max(most, P->nnzb);
     room_for_split(c, s.n_atoms, most, most, true);
   } else if (s.B == 4) {
-    for (const auto& q : s.qcache) most = std::max(most, q.second->P.nnzb);
-    bool any = false;
-    for (const auto& ti : s.tcache) any = any || ti.second->quads;
-    if (any) room_for_split(c, (s.n_atoms + 3) / 4, most, most, true);
+    for (const auto& ti : s.tcache)
+      if (ti.second->qa) most = std::max({most, ti.second->qa->P.nnzb, ti.second->qb->P.nnzb});
+    if (most) room_for_split(c, (s.n_atoms + 3) / 4, most, most, true);
   }
 }
 
 // Whether a product with this triple list takes its quads
-static bool in_quads(const rt_ctx* c, const TripleInfo& ti) { return ti.quads && !c->x_off; }
+static bool in_quads(const rt_ctx* c, const TripleInfo& ti, bool cplx) {
+  return ti.qa && ti.quad_fill >= (cplx ? QUAD_FILL_CPLX : QUAD_FILL_REAL) && !c->x_off;
+}
 
 // keep_a: A is the operand of the product just before, unchanged since, so that its split
 // stands (if that product took the same route, which xa_of says).
@@ -521,7 +579,7 @@ static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cpl
   int B = s.B;
   const Pattern* had = c->xa_of;
   c->xa_of = nullptr;
-  quads = quads && in_quads(c, ti);
+  quads = quads && in_quads(c, ti, cplx);
   const Pattern &pa = quads ? ti.qa->P : *ti.pa, &pb = quads ? ti.qb->P : *ti.pb;
   const bool digits = (B == 13 && c->p.precision == RT_FP64) || quads;
   if (digits && (c->counting ? !c->x_off : room_for_split(c, pa.n_atoms, pa.nnzb, pb.nnzb, cplx))) {
@@ -568,6 +626,14 @@ static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cpl
       [&] { launch_gemm(B, fp32, cplx, ad, bd, epi, g, c->ws); });
 }
 
+// All device memory of the context (the stream is done with it).
+static void release_memory(rt_ctx* c) {
+  for (auto& s : c->sys)
+    for (auto& q : s->qcache)
+      if (q.second) q.second->mem.release_all();
+  c->arena.release_all();
+}
+
 // Device memory needed only inside one set-up routine: taken from the
 // context's allocator and handed back when the routine ends, once the stream
 // has finished with it (the context's arena keeps everything else until
@@ -599,10 +665,11 @@ static GemmArgs args(const void* A, const void* B, void* C) {
 }
 
 // residual ||I - Y||_F / sqrt(n) from the per-item partials of an EPI_TWO_I product
-static void residual_from_items(rt_ctx* c, Sys& s, const TripleInfo& ti, double* out, double* out2) {
+static void residual_from_items(rt_ctx* c, Sys& s, const TripleInfo& ti, bool cplx, double* out, double* out2) {
+  const int64_t n = in_quads(c, ti, cplx) ? ti.qt.n_items : ti.t.n_items;
   run(
       c, PC_MISC, 0, 0,
-      [&] { launch_sum(s.red_items, in_quads(c, ti) ? ti.qt.n_items : ti.t.n_items, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
+      [&] { launch_sum(s.red_items, n, s.red_part, std::sqrt((double)s.n_true), out, out2, c->ws); }, 2);
 }
 
 // ----------------------------------------------------------------------------
@@ -854,6 +921,7 @@ static void setup_system(rt_ctx* c, Sys& s, const rt_system& in) {
       s.planar = p.packed_fma != 0 && !p.tensor_cores;
     }
   }
+  release_quads(s);
   reserve_for_step(c, s);
   RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
 }
@@ -883,7 +951,7 @@ static rt_status hotelling_sinv(rt_ctx* c, Sys& s) {
     GemmArgs g = args(s.S, s.Sinv, s.Zs);
     g.red = s.red_items;
     gemm(c, s, PC_MISC, tSX, false, false, false, false, EPI_TWO_I, g, P);
-    residual_from_items(c, s, tSX, s.scal, nullptr);
+    residual_from_items(c, s, tSX, false, s.scal, nullptr);
     RT_CUDA_CHECK(cudaMemcpyAsync(&res, s.scal, sizeof(double), cudaMemcpyDeviceToHost, c->ws));
     RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
     if (!std::isfinite(res) || res > 1.0) {
@@ -1262,7 +1330,7 @@ static void build_propagator(rt_ctx* c, Sys& s, bool fp32) {
       GemmArgs g = args(s.Acn, xi, s.Zc);
       g.red = s.red_items;
       gemm(c, s, PC_CN_HOT, tAX, false, true, false, false, EPI_TWO_I, g, s.pU);
-      if (it == n64 - 1) residual_from_items(c, s, tAX, s.scal + 1, nullptr);
+      if (it == n64 - 1) residual_from_items(c, s, tAX, true, s.scal + 1, nullptr);
       gemm(c, s, PC_CN_HOT, tXZ, false, true, false, false, EPI_STORE, args(xi, s.Zc, xo), s.pU);
     }
     if (n64 % 2 == 1)
@@ -1891,12 +1959,12 @@ static void unitarity(rt_ctx* c, Sys& s, int metric, double* mx, double* mean) {
   if (s.duf_current)
     launch_u_from_delta(s.dUf, s.U, s.pU->nnzb, s.pU->rowidx, s.pU->col, s.B, c->ws);  // U = I + dU
   if (metric) {
-    TripleInfo& tW = triples_for(c, s, s.pS, false, s.pU, false, s.pW, false);
-    TripleInfo& tE = triples_for(c, s, s.pU, true, s.pW, false, s.pU, false);
+    TripleInfo& tW = triples_for(c, s, s.pS, false, s.pU, false, s.pW, false, false);
+    TripleInfo& tE = triples_for(c, s, s.pU, true, s.pW, false, s.pU, false, false);
     gemm(c, s, PC_MISC, tW, false, true, false, false, EPI_STORE, args(s.Sc, s.U, s.W), s.pW, false, false);
     gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.W, s.E), s.pU, false, false);
   } else {
-    TripleInfo& tE = triples_for(c, s, s.pU, true, s.pU, false, s.pU, false);
+    TripleInfo& tE = triples_for(c, s, s.pU, true, s.pU, false, s.pU, false, false);
     gemm(c, s, PC_MISC, tE, false, true, true, false, EPI_STORE, args(s.U, s.U, s.E), s.pU, false, false);
   }
   double* pmax = c->arena.get_n<double>(1024);
@@ -2212,7 +2280,7 @@ rt_status rt_create(rt_ctx** out, const rt_system* sys, int32_t n_sys, const rt_
     RT_CUDA_CHECK(cudaStreamSynchronize(c->ws));
   } catch (const Error& e) {
     if (c->ws) cudaStreamSynchronize(c->ws);
-    c->arena.release_all();
+    release_memory(c);
     if (c->ws) cudaStreamDestroy(c->ws);
     if (c->ev_in) cudaEventDestroy(c->ev_in);
     if (c->ev_out) cudaEventDestroy(c->ev_out);
@@ -2877,7 +2945,7 @@ void rt_destroy(rt_ctx* c) {
     cudaEventDestroy(e.first);
     cudaEventDestroy(e.second);
   }
-  c->arena.release_all();
+  release_memory(c);
   if (c->ev_in) cudaEventDestroy(c->ev_in);
   if (c->ev_out) cudaEventDestroy(c->ev_out);
   if (c->ws) cudaStreamDestroy(c->ws);

@@ -245,8 +245,9 @@ void launch_gemm13_x64(bool cplx, bool a_dag, bool b_dag, Epilogue epi, const Ge
 struct QuadPattern {
   Pattern P;               // over (n_atoms + 3) / 4 groups
   int32_t* map = nullptr;  // [P.nnzb][4 row atoms][4 column atoms] block of the pattern, -1: none
+  Arena mem;               // what holds both
 };
-void build_quads(QuadPattern& Q, const Pattern& P, Arena& arena, cudaStream_t st);
+void build_quads(QuadPattern& Q, const Pattern& P, cudaStream_t st);
 
 // Launches; `cplx` selects complex values, `b_dag` conj-transposes B's blocks,
 // `a_dag` A's blocks.  Element type by precision: FP64 double/double2, FP32 float/float2.
