@@ -180,12 +180,26 @@ TRAFFIC = {("diamond 4096 atoms x 13 functions, r_S=r_H=7A, r_Sinv=r_T=r_U=r_K=r
 
 
 def derived_alu_peaks(torch, sm_max_mhz):
-    """ALU peaks from unit counts and the maximum SM clock, TFLOP/s: FP32 is
-    128 FMA lanes per SM x 2 flops; FP64 is GB300's nominal 1.25 TFLOP/s at
-    2070 MHz scaled to the clock (2 FP64 FMA per clock per SM on 152 SMs)."""
+    """ALU peak from unit counts and the maximum SM clock, TFLOP/s: FP32 is 128 FMA lanes per SM x 2 flops."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     ghz = (sm_max_mhz or 2070.0) / 1e3
-    return {"fp32": sms * 128 * 2 * ghz / 1e3, "fp64": sms * 2 * 2 * ghz / 1e3, "sms": sms, "sm_max_ghz": ghz}
+    return {"fp32": sms * 128 * 2 * ghz / 1e3, "sms": sms, "sm_max_ghz": ghz}
+
+
+def alu_roofline(path, kernel, flops, ms, derived, cublas, traffic):
+    """The roofline of one launch.  FP64 products of the FP64 path have no peak: they are exact digit products on the
+    tensor cores (mma.sync FP16, 15 to 43 pairs of digits to a product by the digits that its blocks leave at zero), several
+    times the FP64 units' rate."""
+    achieved = flops / (ms / 1e3) / 1e12
+    peak = derived["fp32"] if path == "fp32" else None
+    return {"bound": "alu" if peak else "tensor", "kernel": kernel, "achieved": round(achieved, 3),
+            "peak": round(peak, 3) if peak else None, "unit": "TFLOP/s",
+            "frac": round(achieved / peak, 4) if peak else None, "traffic": traffic,
+            "peak_source": (f"derived: {derived['sms']} SMs x 128 FP32 lanes x 2 flops x {derived['sm_max_ghz']:.3f} GHz"
+                            if peak else "none: exact digit products on the tensor cores, pairs by the data"),
+            "cublas_gemm_tflops": {k: round(v, 3) for k, v in cublas.items()},
+            "frac_of_cublas_gemm": round(achieved / cublas[path], 4) if cublas.get(path) else None,
+            "per_launch_flops": flops, "per_launch_ms": round(ms, 4)}
 
 
 def alu_peaks(torch):
@@ -446,17 +460,8 @@ def run_gpu(args):
     derived = derived_alu_peaks(torch, clk.get("sm_max_mhz") if isinstance(clk, dict) else None)
     mp = measured_peaks()
     if d["flops"] > 0:
-        achieved = per_launch_flops / (per_launch_ms / 1e3) / 1e12
-        peak = derived[hp]
-        roof = {"bound": "alu", "kernel": dom, "achieved": round(achieved, 3), "peak": round(peak, 3),
-                "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
-                "traffic": TRAFFIC.get((cfg_name(args), hp, dom)),
-                "peak_source": (f"derived: {derived['sms']} SMs x "
-                                f"{'128 FP32 lanes x 2 flops' if hp == 'fp32' else '2 FP64 FMA x 2 flops'}"
-                                f" x {derived['sm_max_ghz']:.3f} GHz"),
-                "cublas_gemm_tflops": {k: round(v, 3) for k, v in peaks.items()},
-                "frac_of_cublas_gemm": round(achieved / peaks[hp], 4) if peaks.get(hp) else None,
-                "per_launch_flops": per_launch_flops, "per_launch_ms": round(per_launch_ms, 4)}
+        roof = alu_roofline(hp, dom, per_launch_flops, per_launch_ms, derived, peaks,
+                            TRAFFIC.get((cfg_name(args), hp, dom)))
     else:
         achieved = d["bytes"] / max(d["launches"], 1) / (per_launch_ms / 1e3) / 1e9
         peak = mp.get("hbm_gbs", 6800.0)
