@@ -52,9 +52,9 @@ struct TripleKey {
 struct TripleInfo {
   const Pattern *pa = nullptr, *pb = nullptr;  // the operands' patterns
   Triples t;
-  // FP64 4-function products as quads (16 x 16 blocks of four consecutive atoms): triples to a product of quads,
-  // and, where that is enough for either kind of product, the quads' list and patterns
-  double quad_fill = 0.0;
+  // FP64 4-function products as quads (16 x 16 blocks of four consecutive atoms): triples to a product of quads and
+  // to an output block, and, where these are enough for either kind of product, the quads' list and patterns
+  double quad_fill = 0.0, quad_chain = 0.0;
   bool quads_counted = false;
   Triples qt;
   const QuadPattern *qa = nullptr, *qb = nullptr, *qc = nullptr;
@@ -298,6 +298,12 @@ static Pattern* pattern_for(rt_ctx* c, Sys& s, double r) {
 // 269 / 256 at 6.6, 198 / 192 at 7.3, 573 / 582 at 7.7, 641 / 806 at 7.8, 298 / 372 at 8.8; M = U K 389 / 303 at 4.9,
 // 447 / 464 at 5.9, 839 / 935 at 6.6, 578 / 683 at 7.3.
 constexpr double QUAD_FILL_REAL = 7.5, QUAD_FILL_CPLX = 5.75;
+// And from this many triples to an output block on: in the smallest systems a product lasts as long as the chain of one
+// block's triples (0.5 us a real one, 1 us a complex one), in quads 7 us longer than one triple does.  A captured step of n
+// atoms that all reach one another, us: EM (mostly real) all in quads 76 at 2, 86 at 8 and at 12, 92 at 16, 98 at 20; with the
+// real products on the FP64 pipe 31, 62, 72, 84 and (by the slope) 99; CN (all complex) in quads 101 at 6, 105 at 8, 107
+// at 10; on the FP64 pipe 80, 103 and 123.
+constexpr double QUAD_CHAIN_REAL = 20, QUAD_CHAIN_CPLX = 8;
 
 // The quads of a triple list, where there are triples enough to a product of them.  Patterns that no list takes are given
 // back by release_quads.
@@ -336,12 +342,14 @@ static void add_quads(rt_ctx* c, Sys& s, TripleInfo& ti, const TripleKey& k) {
     return;  // no memory for them: the CUDA-core products need none
   }
   const double fill = qt.n_triples ? (double)ti.t.n_triples / (double)qt.n_triples : 0.0;
-  if (fill < std::min(QUAD_FILL_REAL, QUAD_FILL_CPLX)) {
+  const double chain = ti.t.n_items ? (double)ti.t.n_triples / (double)ti.t.n_items : 0.0;
+  if (fill < std::min(QUAD_FILL_REAL, QUAD_FILL_CPLX) || chain < std::min(QUAD_CHAIN_REAL, QUAD_CHAIN_CPLX)) {
     list.release_all();
     return;
   }
   c->arena.blocks.insert(c->arena.blocks.end(), list.blocks.begin(), list.blocks.end());
   ti.quad_fill = fill;
+  ti.quad_chain = chain;
   ti.qt = qt;
   ti.qa = qa;
   ti.qb = qb;
@@ -564,7 +572,8 @@ static void reserve_for_step(rt_ctx* c, Sys& s) {
 
 // Whether a product with this triple list takes its quads
 static bool in_quads(const rt_ctx* c, const TripleInfo& ti, bool cplx) {
-  return ti.qa && ti.quad_fill >= (cplx ? QUAD_FILL_CPLX : QUAD_FILL_REAL) && !c->x_off;
+  return ti.qa && ti.quad_fill >= (cplx ? QUAD_FILL_CPLX : QUAD_FILL_REAL) &&
+         ti.quad_chain >= (cplx ? QUAD_CHAIN_CPLX : QUAD_CHAIN_REAL) && !c->x_off;
 }
 
 // keep_a: A is the operand of the product just before, unchanged since, so that its split

@@ -45,29 +45,55 @@ def test_lists_of_quads_are_kept_where_they_are_taken(rt, prop, radius, quads):
     assert fp64[1] - fp64[0] == mixed[1] - mixed[0]
 
 
-@pytest.mark.parametrize("cell,radius", [(3, 7.5), (3, 8.0), (4, 7.0), (4, 7.5)])
+# n atoms that all reach one another: n triples to a block
+@pytest.mark.parametrize("n,quads", [(2, False), (7, False), (8, True), (20, True)])
+def test_smallest_systems_take_no_quads(rt, n, quads):
+    from test_gpu_x64_range import _chain
+    H = np.random.default_rng(n).normal(size=(4 * n, 4 * n))
+    s, _ = _chain(H + H.T, 4, 0.1)
+    lists = []
+    for precision in ("fp32", "fp64"):
+        ctx = rt.RT(s, prop="em", dt=0.05, precision=precision, **_radii(6.0))
+        lists.append(ctx.debug_check())
+        ctx.close()
+    assert (lists[1] > lists[0]) == quads
+
+
+@pytest.mark.parametrize("cell,radius", [(3, 7.5), (3, 8.0), (4, 7.0), (4, 7.5), (0, 9), (0, 21)])
+# cell 0: 9 or 21 atoms that all reach one another
 @pytest.mark.parametrize("prop", ["em", "cn"])
 def test_quads_agree_with_the_cuda_cores(rt, monkeypatch, prop, cell, radius):
     from test_gpu_memory import Limited
-    s = _system(cell)
+    from test_gpu_x64_range import _chain
+    if cell:
+        s = _system(cell)
+    else:
+        H = np.random.default_rng(0).normal(size=(4 * radius, 4 * radius))
+        s, _ = _chain(H + H.T, 4, 0.1)
     rng = np.random.default_rng(1)
 
-    def trajectory(limit):
-        mem = Limited(rt, limit)
-        monkeypatch.setattr(rt, "_torch_allocator", lambda: mem.hooks)
-        ctx = rt.RT(s, prop=prop, dt=0.05, **_radii(radius))
+    def trajectory(refused):
+        mem = Limited(rt)
+        get = lambda n, stream, user: None if n == refused else mem.hooks[0](n, stream, user)
+        hooks = rt.ALLOC_FN(get), mem.hooks[1]
+        monkeypatch.setattr(rt, "_torch_allocator", lambda: hooks)
+        ctx = rt.RT(s, prop=prop, dt=0.01, **_radii(max(radius, 6.0) if cell else 6.0))
         ctx.inverse()
-        ctx.set_density(0, 0, K0)
+        rowptr, col = ctx.pattern(0, rt.RT_PAT_U)
+        K0 = rng.normal(size=16 * len(col)) + 1j * rng.normal(size=16 * len(col))
+        ctx.set_density(0, 0, K0 if refused is None else out["K0"])
         ctx.step(2)
-        out = [ctx.matrix(0, m) for m in (rt.RT_MAT_SINV, rt.RT_MAT_U, rt.RT_MAT_K)]
+        got = [ctx.matrix(0, m) for m in (rt.RT_MAT_SINV, rt.RT_MAT_U, rt.RT_MAT_K)]
         ctx.close()
-        return out, mem
+        rows = np.repeat(np.arange(s.n_atoms), np.diff(rowptr))
+        blocks = len(set(zip((rows // 4).tolist(), (col // 4).tolist())))
+        out.setdefault("K0", K0)
+        return got, mem, (8192 * blocks + 16 + 255) // 256 * 256  # the digits of one split operand
 
-    probe = rt.RT(s, prop=prop, dt=0.05, **_radii(radius))
-    n = 16 * len(probe.pattern(0, rt.RT_PAT_K)[1])
-    probe.close()
-    K0 = rng.normal(size=n) + 1j * rng.normal(size=n)
-    with_quads, mem = trajectory(None)
-    without, _ = trajectory(mem.peak - sum(sorted(mem.sizes)[-2:]))
+    out = {}
+    with_quads, mem, digits = trajectory(None)
+    assert digits in mem.sizes
+    without, mem, _ = trajectory(digits)
+    assert digits not in mem.sizes
     for a, b in zip(with_quads, without):  # either route rounds a product to 2^-53 of a few hundred terms
         assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()

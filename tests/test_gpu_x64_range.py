@@ -77,14 +77,14 @@ def _signs(rng, shape):
     return rng.choice([-1.0, 1.0], size=shape)
 
 
-# 4-function systems go in quads of four atoms: with and without a last group of fewer
-@pytest.mark.parametrize("b,n", [(13, 1), (13, 9), (4, 8), (4, 9), (4, 30)])
+# 4-function systems of 20 atoms and more go in quads of four: with and without a last group of fewer
+@pytest.mark.parametrize("b,n", [(13, 1), (13, 9), (4, 20), (4, 21), (4, 45)])
 def test_product_with_the_identity_of_graded_entries(rt, b, n):
     rng = np.random.default_rng(b * n)
     N = b * n
     H = rng.uniform(0.5, 1.0, (N, N)) * _signs(rng, (N, N)) * 2.0 ** -rng.integers(0, 41, (N, N)).astype(float)
     H *= 2.0 ** rng.integers(-30, 31, N).astype(float)  # one scale per column
-    s, near = _chain(H, b, 0.3)
+    s, near = _chain(H, b, 0.2)
     ctx = rt.RT(s, prop="em", dt=0.05, **RADII)
     ctx.inverse()
     ctx.propagator(0.0)
@@ -110,7 +110,7 @@ def _square(rt, T, b, spacing):
 
 
 @pytest.mark.parametrize("grade", [0, 7, 14])
-@pytest.mark.parametrize("b,n", [(13, 1), (13, 2), (13, 3), (13, 9), (4, 5), (4, 8), (4, 33)])
+@pytest.mark.parametrize("b,n", [(13, 1), (13, 2), (13, 3), (13, 9), (4, 22), (4, 24), (4, 33)])
 def test_every_element_of_a_graded_product(rt, b, n, grade):
     """T = D^-1 R D with D = 2^0..2^grade: the elements of T T span 2^+-grade, their terms one power of two each.
     A term is off by at most 2 2^(grade + 1) 2^-71 2^2 of itself (|R| in [0.5, 1)), at most 2^-53 for grade 14; the sum's one
@@ -125,7 +125,7 @@ def test_every_element_of_a_graded_product(rt, b, n, grade):
     assert (err <= 4.0 * 2.0 ** -53 * (np.abs(T) @ np.abs(T)))[off].all()
 
 
-@pytest.mark.parametrize("b,n", [(13, 1), (13, 2), (13, 9), (13, 40), (4, 9), (4, 60)])
+@pytest.mark.parametrize("b,n", [(13, 1), (13, 2), (13, 9), (13, 40), (4, 21), (4, 60)])
 def test_sums_of_extreme_digits_are_exact(rt, b, n):
     """Every entry the same, its digits -64 and six times -256: the sums of a weight come as close to 2^24 between two
     carries as operands of 53 bits can bring them."""
@@ -139,12 +139,12 @@ def test_sums_of_extreme_digits_are_exact(rt, b, n):
 
 
 @pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
-@pytest.mark.parametrize("b,n", [(13, 3), (4, 9)])
+@pytest.mark.parametrize("b,n", [(13, 3), (4, 21)])
 def test_entries_that_are_not_finite_stay_in_their_column(rt, b, n, bad):
     rng = np.random.default_rng(7)
     H = rng.uniform(0.5, 1.0, (b * n, b * n))
     H[1, b + 2] = bad
-    s, near = _chain(H, b, 0.3)
+    s, near = _chain(H, b, 0.2)
     ctx = rt.RT(s, prop="em", dt=0.05, **RADII)
     ctx.inverse()
     ctx.propagator(0.0)
