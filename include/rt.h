@@ -109,7 +109,9 @@ enum {
 };
 
 /* Device allocator hook: return `bytes` of device memory usable on `stream`, or
- * NULL on failure.  The free hook gets the same pointer back. */
+ * NULL on failure.  The free hook gets the same pointer back.  A refused request
+ * may be followed by frees and the same request again, and an FP64 context goes
+ * on without the split copies of its operands (slower) where they are refused. */
 typedef void* (*rt_alloc_fn)(size_t bytes, void* stream, void* user);
 typedef void (*rt_free_fn)(void* ptr, void* stream, void* user);
 
@@ -144,7 +146,10 @@ typedef struct {
                                reductions and the last CN iteration in FP64;
                                EM, ETRS and M4 build U - I in FP32 from
                                T(t) = S^-1 H0 - E(t) S^-1 D, both cut to r_T
-                               and formed once in FP64)                          */
+                               and formed once in FP64).  RT_FP64 multiplies in
+                               72-bit fixed point under one scale per row and
+                               column: basis functions of an atom should have
+                               norms within a few powers of two of each other    */
   int32_t full_step;        /* 1: rebuild U for every step; 0: reuse U            */
   int32_t n_kick;           /* density matrices per system sharing U (1..3)       */
   int32_t kick_terms;       /* Taylor terms of the kick exponential               */

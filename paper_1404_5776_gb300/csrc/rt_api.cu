@@ -593,7 +593,7 @@ static void gemm(rt_ctx* c, Sys& s, int cls, TripleInfo& ti, bool fp32, bool cpl
   const bool digits = (B == 13 && c->p.precision == RT_FP64) || quads;
   if (digits && (c->counting ? !c->x_off : room_for_split(c, pa.n_atoms, pa.nnzb, pb.nnzb, cplx))) {
     // products of the FP64 mode: exact digit products on the tensor cores, of 13-function blocks (6x
-    // the CUDA cores at every size measured, 64 to 512 atoms) and of quads of 4-function blocks;
+    // the CUDA cores at every size measured from 8 to 512 atoms, 1.2x at one atom) and of quads of 4-function blocks;
     // the mixed modes' FP64 set-up keeps its sums (spgemm.cu)
     const int32_t *ma = quads ? ti.qa->map : nullptr, *mb = quads ? ti.qb->map : nullptr,
                   *mc = quads ? ti.qc->map : nullptr;

@@ -48,7 +48,7 @@
 // 16 warps a SM; a warp with both halves (168 registers, 12 warps) measured 1.3
 // times slower.  What bounds it: the tensor pipe, with the wait for the next blocks'
 // first digits and the carries beside it.  216 atoms x 13, r = 8 A: a Taylor power
-// 1.15 ms with its splits 1.20, M = U K 2.80 ms (the CUDA-core kernel: 8.9 and 21.7 ms);
+// 1.15 ms with its splits 1.20, M = U K 3.9 ms, 2.8 for a real K (the CUDA-core kernel: 8.9 and 21.7 ms);
 // FP64 EM step at 512 atoms 22 ms (126).  The time follows the warps in flight: A's
 // digits in two sets of registers (12 warps) took 27 % longer, five CTAs of 96
 // registers (spills) 65 %.
